@@ -1799,10 +1799,10 @@ tt_status tt_kernel_normalize(tt_ctx *ctx, double *d_Ks, double *d_Kxi, double *
 namespace {
 
 // The tables of the inversion grids of mg on the device, rebuilt when mg changes: Wr, Wt, Wp
-// (double) then lo for r, theta, phi (int).
+// (double), then lo for r, theta, phi and the phi nodes under each phi hat (int).
 struct MgTabs {
     const double *Wr, *Wt, *Wp;
-    const int *lo;
+    const int *lo, *rng;
 };
 
 tt_status mgrid_tables(tt_ctx *ctx, const tt_mgrid *mg, MgDims &d, MgTabs &tb) {
@@ -1813,13 +1813,14 @@ tt_status mgrid_tables(tt_ctx *ctx, const tt_mgrid *mg, MgDims &d, MgTabs &tb) {
     const GridC &g = ctx->g;
     d = MgDims{g.nr, g.nt, g.np, mg->n_r, mg->n_t, mg->n_p, mg->n_grids};
     const size_t nw = (size_t)d.H * ((size_t)d.cr * d.nr + (size_t)d.ct * d.nt + (size_t)d.cp * d.np);
-    const size_t nl = (size_t)d.H * ((size_t)d.nr + d.nt + d.np);
-    ENSURE(ctx->mg_tab, sizeof(double) * nw + sizeof(int) * nl);
+    const size_t nl = (size_t)d.H * ((size_t)d.nr + d.nt + d.np), nr2 = (size_t)d.H * d.cp * 2;
+    ENSURE(ctx->mg_tab, sizeof(double) * nw + sizeof(int) * (nl + nr2));
     double *W = (double *)ctx->mg_tab.p;
     tb.Wr = W;
     tb.Wt = W + (size_t)d.H * d.cr * d.nr;
     tb.Wp = tb.Wt + (size_t)d.H * d.ct * d.nt;
     tb.lo = (const int *)(W + nw);
+    tb.rng = tb.lo + nl;
     const int key[4] = {mg->n_r, mg->n_t, mg->n_p, mg->n_grids};
     if (memcmp(key, ctx->mg_key, sizeof key) == 0) return TT_OK;
     std::vector<double> hw, w;
@@ -1830,9 +1831,20 @@ tt_status mgrid_tables(tt_ctx *ctx, const tt_mgrid *mg, MgDims &d, MgTabs &tb) {
         hw.insert(hw.end(), w.begin(), w.end());
         hl.insert(hl.end(), l.begin(), l.end());
     }
+    // w now holds the phi axis: the nodes under each hat (its weights elsewhere are zero)
+    for (int q = 0; q < d.H * d.cp; ++q) {
+        int k0 = d.np, k1 = 0;
+        for (int k = 0; k < d.np; ++k)
+            if (w[(size_t)q * d.np + k] != 0.0) {
+                k0 = k < k0 ? k : k0;
+                k1 = k + 1;
+            }
+        hl.push_back(k0 < k1 ? k0 : 0);
+        hl.push_back(k1);
+    }
     CK(cudaStreamSynchronize(ctx->st));   // the previous tables may still be read
     CK(cudaMemcpy(W, hw.data(), sizeof(double) * nw, cudaMemcpyHostToDevice));
-    CK(cudaMemcpy(W + nw, hl.data(), sizeof(int) * nl, cudaMemcpyHostToDevice));
+    CK(cudaMemcpy(W + nw, hl.data(), sizeof(int) * (nl + nr2), cudaMemcpyHostToDevice));
     memcpy(ctx->mg_key, key, sizeof key);
     return TT_OK;
 }
@@ -1853,7 +1865,7 @@ tt_status tt_mgrid_project(tt_ctx *ctx, const tt_mgrid *mg, const double *d_K, d
     double *T1 = (double *)ctx->mg_scr.p;
     const GridC &g = ctx->g;
     CK(run_mgrid_project(d, d_K, ctx->gd.h2, ctx->gd.cost, g.dr * g.dt * g.dp, tb.Wr, tb.Wt,
-                         tb.Wp, T1, T1 + n1, d_G, ctx->st));
+                         tb.Wp, tb.rng, T1, T1 + n1, d_G, ctx->st));
     ctx->launches += 3;
     return TT_OK;
 }
@@ -1865,8 +1877,9 @@ tt_status tt_mgrid_expand(tt_ctx *ctx, const tt_mgrid *mg, const double *d_G, do
     MgTabs tb;
     tt_status s;
     if ((s = mgrid_tables(ctx, mg, d, tb)) != TT_OK) return s;
-    CK(run_mgrid_expand(d, d_G, tb.lo, tb.Wr, tb.Wt, tb.Wp, d_D, ctx->st));
-    ctx->launches += 1;
+    ENSURE(ctx->mg_scr, sizeof(double) * (size_t)d.H * d.nr * d.nt * d.cp);
+    CK(run_mgrid_expand(d, d_G, tb.lo, tb.Wr, tb.Wt, tb.Wp, (double *)ctx->mg_scr.p, d_D, ctx->st));
+    ctx->launches += 2;
     return TT_OK;
 }
 
@@ -1878,7 +1891,7 @@ tt_status tt_kernel_normalize_rel(tt_ctx *ctx, double *d_Ks, double *d_Kxi, doub
     if (!(eps_rel > 0) || !(zeta >= 0))
         return fail(ctx, TT_EINVAL, "tt_kernel_normalize_rel: eps_rel must be > 0 and zeta >= 0");
     constexpr int kParts = 304;
-    ENSURE(ctx->upd_part, sizeof(double) * (3 * kParts + 3));
+    ENSURE(ctx->upd_part, sizeof(double) * (3 * kParts + 6));
     CK(run_kernel_normalize_rel(ctx->g.N, d_Ks, d_Kxi, d_Keta, d_Kd, eps_rel, zeta,
                                 (double *)ctx->upd_part.p, kParts, ctx->st));
     ctx->launches += 3;
@@ -1891,7 +1904,7 @@ tt_status tt_misfit_total(tt_ctx *ctx, int n_src, const double *d_chi, double al
     if (!d_chi || !h_total || n_src < 1 || n_src > TT_MAX_BATCH)
         return fail(ctx, TT_EINVAL, "tt_misfit_total: NULL argument or n_src outside 1..%d",
                     TT_MAX_BATCH);
-    ENSURE(ctx->upd_part, sizeof(double) * (3 * 304 + 3));
+    ENSURE(ctx->upd_part, sizeof(double) * (3 * 304 + 6));
     double *d_out = (double *)ctx->upd_part.p;
     CK(run_misfit_total(n_src, d_chi, alpha, beta, d_chi_cr, gamma, d_out, ctx->st));
     ctx->launches += 1;
@@ -1910,7 +1923,7 @@ tt_status tt_model_update(tt_ctx *ctx, const tt_model *model, const double *d_Ds
     if (!d_Ds || !d_Dxi || !d_Deta) return fail(ctx, TT_EINVAL, "tt_model_update: NULL direction");
     if (!(step > 0) || !(step < 1)) return fail(ctx, TT_EINVAL, "tt_model_update: step must be in (0, 1)");
     constexpr int kParts = 304;   // 2 x 152 SMs
-    ENSURE(ctx->upd_part, sizeof(double) * (3 * kParts + 3));
+    ENSURE(ctx->upd_part, sizeof(double) * (3 * kParts + 6));
     double *part = (double *)ctx->upd_part.p;
     const long long N = ctx->g.N;
     if (model->dtype == TT_F32)

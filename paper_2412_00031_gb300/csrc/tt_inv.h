@@ -29,16 +29,18 @@ cudaError_t run_kernel_density(long long N, int B, const F *P, double *Kd, cudaS
 cudaError_t run_kernel_normalize(long long N, double *Ks, double *Kxi, double *Keta,
                                  const double *Kd, double eps, double zeta, cudaStream_t st);
 // Eq. 17: G[h][a][b][c] for one kernel K; T1 ([H][nr][nt][cp]) and T2 ([H][nr][ct][cp]) are
-// scratch; dV = h2[i]^2 cost[j] dvol.
+// scratch; dV = h2[i]^2 cost[j] dvol; rng[h][c] = [first, end) of the phi nodes under hat c.
 cudaError_t run_mgrid_project(const MgDims &d, const double *K, const double *h2,
                               const double *cost, double dvol, const double *Wr,
-                              const double *Wt, const double *Wp, double *T1, double *T2,
-                              double *G, cudaStream_t st);
-// Eq. 15: D at the forward nodes from the coefficients G; lo = the three axes' lo tables.
+                              const double *Wt, const double *Wp, const int *rng, double *T1,
+                              double *T2, double *G, cudaStream_t st);
+// Eq. 15: D at the forward nodes from the coefficients G; lo = the three axes' lo tables; E
+// ([H][nr][nt][cp]) is scratch.
 cudaError_t run_mgrid_expand(const MgDims &d, const double *G, const int *lo, const double *Wr,
-                             const double *Wt, const double *Wp, double *D, cudaStream_t st);
+                             const double *Wt, const double *Wp, double *E, double *D,
+                             cudaStream_t st);
 // Eq. 18 with eps = eps_rel max(Kd), the maximum taken on the device; part: scratch of
-// 3 n_part + 3 doubles.
+// 3 n_part + 6 doubles.
 cudaError_t run_kernel_normalize_rel(long long N, double *Ks, double *Kxi, double *Keta,
                                      const double *Kd, double eps_rel, double zeta, double *part,
                                      int n_part, cudaStream_t st);
@@ -46,7 +48,7 @@ cudaError_t run_kernel_normalize_rel(long long N, double *Ks, double *Kxi, doubl
 // FP64 in a fixed order.
 cudaError_t run_misfit_total(int n, const double *chi, double alpha, double beta,
                              const double *chi_cr, double gamma, double *out, cudaStream_t st);
-// The model update; part: scratch of 3 n_part + 3 doubles.
+// The model update; part: scratch of 3 n_part + 6 doubles.
 template <typename F>
 cudaError_t run_model_update(long long N, F *s, F *xi, F *eta, const double *Ds,
                              const double *Dxi, const double *Deta, double step, double *part,

@@ -68,8 +68,9 @@ struct tt_ctx {
     DevBuf ord_perm, ord_pts, ord_src, ord_tabT, ord_tabP, ord_tau, ord_iters, ord_conv;
     // inversion step: multiple-grid tables (for mg_key), projection scratch, update scratch
     DevBuf mg_tab, mg_scr, upd_part;
-    // teleseismic events: 2-D tau scratch, event radii / coordinates and iteration counts
-    DevBuf tele_tau, tele_aux;
+    // teleseismic events: 2-D tau scratch, event radii / coordinates and iteration counts, the
+    // 2-D nodes' constants
+    DevBuf tele_tau, tele_aux, tele_pre;
     int mg_key[4] = {0, 0, 0, 0};
     struct Tuned { int n_src, dtype, scheme, schedule, groups; };
     std::vector<Tuned> tuned;
@@ -1300,7 +1301,7 @@ void tt_ctx_destroy(tt_ctx *ctx) {
                       &ctx->net_wt, &ctx->net_part, &ctx->net_scr, &ctx->tune_tau, &ctx->tau_w,
                       &ctx->slot_srcc, &ctx->slot_int,
                       &ctx->net_wbf, &ctx->mg_tab, &ctx->mg_scr, &ctx->upd_part,
-                      &ctx->tele_tau, &ctx->tele_aux, &ctx->net_img, &ctx->net_timg,
+                      &ctx->tele_tau, &ctx->tele_aux, &ctx->tele_pre, &ctx->net_img, &ctx->net_timg,
                       &ctx->net_rows, &ctx->ord_perm, &ctx->ord_pts, &ctx->ord_src,
                       &ctx->ord_tabT, &ctx->ord_tabP, &ctx->ord_tau, &ctx->ord_iters,
                       &ctx->ord_conv};
@@ -1579,10 +1580,13 @@ tt_status tt_tele2d(tt_ctx *ctx, int dtype, int n_r, int n_d, double r_min_km, d
     CK(cudaMemcpyAsync(d_rs, h_r_src_km, sizeof(double) * n_ev, cudaMemcpyHostToDevice, ctx->st));
     const double dr = (r_max_km - r_min_km) / (n_r - 1);
     const double dd = d_max_deg * (3.14159265358979323846 / 180.0) / (n_d - 1);
+    // the nodes' constants, where they fit: the solve runs without them too
+    void *pre = ensure(ctx, ctx->tele_pre, 4 * fs * (size_t)n_ev * n_r * n_d) == TT_OK ? ctx->tele_pre.p
+                                                                                       : nullptr;
     CK(dtype == TT_F32 ? run_tele2d<float>(n_r, n_d, r_min_km, dr, dd, d_s_r, d_rs, n_ev, tol,
-                                           max_iter, ctx->tele_tau.p, d_T, d_it, ctx->st)
+                                           max_iter, ctx->tele_tau.p, pre, d_T, d_it, ctx->n_sm, ctx->st)
                        : run_tele2d<double>(n_r, n_d, r_min_km, dr, dd, d_s_r, d_rs, n_ev, tol,
-                                            max_iter, ctx->tele_tau.p, d_T, d_it, ctx->st));
+                                            max_iter, ctx->tele_tau.p, pre, d_T, d_it, ctx->n_sm, ctx->st));
     ctx->launches += 1;
     std::vector<int> it(n_ev);
     CK(cudaMemcpyAsync(it.data(), d_it, sizeof(int) * n_ev, cudaMemcpyDeviceToHost, ctx->st));

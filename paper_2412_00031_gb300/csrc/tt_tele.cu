@@ -9,8 +9,10 @@
 // mirror; the faces r = r_min, r = r_max and Delta = Delta_max take tau_0 = max(2 tau_1 -
 // tau_2, tau_2) after each sweep; the 3 x 2 nodes next to the event keep tau = 1. The four
 // orderings sweep the anti-diagonals of the (r, Delta) grid, which gives the lexicographic
-// order's result for this five-point stencil. One block per event: its sweeps need only
-// block barriers, and every loop is bounded by max_iter.
+// order's result for this five-point stencil. One block per event, or a cluster of blocks where
+// the events leave SMs idle: the sweeps need only block or cluster barriers, and every loop is
+// bounded by max_iter.
+#include <cooperative_groups.h>
 #include <cuda_runtime.h>
 
 #include "tt_common.cuh"
@@ -20,7 +22,8 @@ namespace ttgb {
 
 namespace {
 
-constexpr int kTeleThreads = 512;
+constexpr int kTeleThreads = 512;   // of an event, over the blocks of its cluster
+constexpr int kTeleCluster = 8;
 
 template <typename F>
 __device__ __forceinline__ F s_of_r(int n_r, F r_min, F dr, const F *s_r, F r) {
@@ -49,13 +52,22 @@ __device__ __forceinline__ void chord(F r, F r_s, F D, F &L2, F &ur, F &ud) {
     ud = mul_(mul_(r_s, sin_(D)), inv);
 }
 
+// What the update of a node takes from its place alone: u = grad T0 / T0, the squared right-hand
+// side (s / (s_s L))^2 and e_D = 1 / (r dD). Two sines, three divisions and a root.
 template <typename F>
-__device__ F god2d(F r, F D, F r_s, F s_s, F s_here, F dr, F dd, F tc, F lo0, F hi0, F lo1,
-                   F hi1) {
+__device__ __forceinline__ Vec4<F> node_consts(int n_r, F r_min, F dr, F dd, const F *s_r, F r_s,
+                                               F s_s, int i, int j) {
+    const F r = fma_((F)i, dr, r_min), D = mul_((F)j, dd);
     F L2, u0, u1;
     chord<F>(r, r_s, D, L2, u0, u1);
-    const F u[2] = {u0, u1};
-    const F e[2] = {div_((F)1, dr), div_((F)1, mul_(r, dd))};
+    const F rhs = div_(s_of_r<F>(n_r, r_min, dr, s_r, r), mul_(s_s, sqrt_(L2)));
+    return Vec4<F>{u0, u1, mul_(rhs, rhs), div_((F)1, mul_(r, dd))};
+}
+
+template <typename F>
+__device__ F god2d(const Vec4<F> &q, F e0, F tc, F lo0, F hi0, F lo1, F hi1) {
+    const F u[2] = {q.x, q.y};
+    const F e[2] = {e0, q.w};
     const F lo[2] = {lo0, lo1}, hi[2] = {hi0, hi1};
     F a[2], c[2], sg[2];
 #pragma unroll
@@ -66,8 +78,7 @@ __device__ F god2d(F r, F D, F r_s, F s_s, F s_here, F dr, F dd, F tc, F lo0, F 
         a[d] = add_(se, u[d]);
         c[d] = fma_(u[d], tc, mul_(se, sub_(tc, lower ? lo[d] : hi[d])));
     }
-    const F rhs = div_(s_here, mul_(s_s, sqrt_(L2)));
-    const F r2 = mul_(rhs, rhs);
+    const F r2 = q.z;
     F bestN = (F)0, bestD = (F)1;
     bool found = false;
     // both axes first: a causal root there is the smallest (each single axis's form never
@@ -104,23 +115,42 @@ __device__ F god2d(F r, F D, F r_s, F s_s, F s_here, F dr, F dd, F tc, F lo0, F 
     return found ? add_(tc, div_(bestN, bestD)) : tc;
 }
 
-template <typename F>
-__global__ void __launch_bounds__(kTeleThreads)
+// PRE: the constants of every node are computed once and kept in `pre` [n_ev][n_r][n_d]; in FP64
+// they are three quarters of an update's instructions on a pipe of 2 lanes a clock and SM, and an
+// iteration updates a node four times (24 events of 201 x 401 nodes with the region's 81x101x101
+// solve: 1129 -> 674 ms, with the clusters below). Without it (no memory for `pre`) every update computes
+// them; the bits are the same.
+// CL: blocks of an event. A diagonal of a few hundred nodes keeps one SM's FP64 pipe busy for a few
+// microseconds; spread over a cluster it costs little more than the barrier.
+template <typename F, bool PRE, int CL>
+__global__ void __launch_bounds__(kTeleThreads / (CL > 4 ? 4 : CL))
 tele2d_kernel(int n_r, int n_d, F r_min, F dr, F dd, const F *s_r, const double *r_src,
-              F tol, int max_iter, F *tau_all, F *T_all, int *iters) {
-    __shared__ F red[kTeleThreads];
-    __shared__ int done;
-    const int ev = blockIdx.x;
-    const int tid = threadIdx.x;
+              F tol, int max_iter, F *tau_all, Vec4<F> *pre_all, F *T_all, int *iters) {
+    namespace cg = cooperative_groups;
+    constexpr int TB = kTeleThreads / (CL > 4 ? 4 : CL);   // threads of a block
+    constexpr int TE = TB * CL;                             // threads of an event
+    __shared__ F red[TB];
+    __shared__ F part[kTeleCluster];                        // the first block's: every block's maximum
+    const int ev = blockIdx.x / CL, rank = blockIdx.x % CL;
+    const int lt = threadIdx.x;
+    const int tid = lt * CL + rank;   // neighbouring nodes of a diagonal on different blocks
+    auto sync = [&]() {
+        if constexpr (CL > 1) cg::this_cluster().sync();
+        else __syncthreads();
+    };
     const long long NN = (long long)n_r * n_d;
     F *tau = tau_all + ev * NN;
     const F r_s = (F)r_src[ev];
     const F s_s = s_of_r<F>(n_r, r_min, dr, s_r, r_s);
     int is = (int)floor((double)((r_s - r_min) / dr) + 0.5);
     is = is < 0 ? 0 : (is > n_r - 1 ? n_r - 1 : is);
-    for (long long q = tid; q < NN; q += kTeleThreads) tau[q] = (F)1;
-    if (tid == 0) done = 0;
-    __syncthreads();
+    Vec4<F> *pre = pre_all + (PRE ? ev * NN : 0);
+    const F e0 = div_((F)1, dr);
+    for (long long q = tid; q < NN; q += TE) {
+        tau[q] = (F)1;
+        if (PRE) pre[q] = node_consts<F>(n_r, r_min, dr, dd, s_r, r_s, s_s, (int)(q / n_d), (int)(q % n_d));
+    }
+    sync();
     int it = 0;
     for (; it < max_iter; ++it) {
         F err = (F)0;
@@ -130,24 +160,23 @@ tele2d_kernel(int n_r, int n_d, F r_min, F dr, F dd, const F *s_r, const double 
             for (int L = 0; L <= na + nb - 2; ++L) {
                 const int a0 = L - (nb - 1) > 0 ? L - (nb - 1) : 0;
                 const int a1 = L < na - 1 ? L : na - 1;
-                for (int a = a0 + tid; a <= a1; a += kTeleThreads) {
+                for (int a = a0 + tid; a <= a1; a += TE) {
                     const int b = L - a;
                     const int i = up_i ? 1 + a : n_r - 2 - a;
                     const int j = up_j ? b : n_d - 2 - b;
                     if (abs(i - is) <= 1 && j <= 1) continue;
                     const long long c = (long long)i * n_d + j;
-                    const F r = fma_((F)i, dr, r_min), D = mul_((F)j, dd);
                     const F tc = tau[c];
-                    const F v = god2d<F>(r, D, r_s, s_s, s_of_r<F>(n_r, r_min, dr, s_r, r), dr,
-                                         dd, tc, tau[c - n_d], tau[c + n_d],
+                    const Vec4<F> k = PRE ? pre[c] : node_consts<F>(n_r, r_min, dr, dd, s_r, r_s, s_s, i, j);
+                    const F v = god2d<F>(k, e0, tc, tau[c - n_d], tau[c + n_d],
                                          tau[(long long)i * n_d + (j > 0 ? j - 1 : 1)], tau[c + 1]);
                     err = fmax(err, fabs(v - tc));
                     tau[c] = v;
                 }
-                __syncthreads();
+                sync();
             }
             // faces r = r_min and r = r_max (all Delta), then Delta = Delta_max (all r)
-            for (int j = tid; j < n_d; j += kTeleThreads) {
+            for (int j = tid; j < n_d; j += TE) {
                 if (!(abs(0 - is) <= 1 && j <= 1))
                     tau[j] = fmax(2 * tau[n_d + j] - tau[2 * n_d + j], tau[2 * n_d + j]);
                 if (!(abs(n_r - 1 - is) <= 1 && j <= 1)) {
@@ -155,30 +184,36 @@ tele2d_kernel(int n_r, int n_d, F r_min, F dr, F dd, const F *s_r, const double 
                     tau[(long long)(n_r - 1) * n_d + j] = fmax(2 * tau[t1] - tau[t2], tau[t2]);
                 }
             }
-            __syncthreads();
-            for (int i = tid; i < n_r; i += kTeleThreads) {
+            sync();
+            for (int i = tid; i < n_r; i += TE) {
                 const long long row = (long long)i * n_d;
                 tau[row + n_d - 1] = fmax(2 * tau[row + n_d - 2] - tau[row + n_d - 3], tau[row + n_d - 3]);
             }
+            sync();
+        }
+        // the event's maximum of the iteration's changes
+        red[lt] = err;
+        __syncthreads();
+        for (int s = TB / 2; s > 0; s >>= 1) {
+            if (lt < s) red[lt] = fmax(red[lt], red[lt + s]);
             __syncthreads();
         }
-        // block maximum of the iteration's changes (fixed order)
-        red[tid] = err;
-        __syncthreads();
-        for (int s = kTeleThreads / 2; s > 0; s >>= 1) {
-            if (tid < s) red[tid] = fmax(red[tid], red[tid + s]);
-            __syncthreads();
+        F m = red[0];
+        if constexpr (CL > 1) {
+            F *p0 = cg::this_cluster().map_shared_rank(part, 0);
+            if (lt == 0) p0[rank] = m;
+            sync();
+#pragma unroll
+            for (int c = 0; c < CL; ++c) m = fmax(m, p0[c]);
         }
-        if (tid == 0) done = red[0] < tol;
-        __syncthreads();
-        if (done) {
+        sync();   // every block has read the maxima
+        if (m < tol) {
             ++it;
             break;
         }
-        __syncthreads();
     }
     if (tid == 0) iters[ev] = it;
-    for (long long q = tid; q < NN; q += kTeleThreads) {
+    for (long long q = tid; q < NN; q += TE) {
         const int i = (int)(q / n_d), j = (int)(q % n_d);
         F L2, u0, u1;
         chord<F>(fma_((F)i, dr, r_min), r_s, mul_((F)j, dd), L2, u0, u1);
@@ -245,13 +280,47 @@ cudaError_t run_tele_shift(long long N, int n_ev, void *T, void *c, int sign, cu
 template cudaError_t run_tele_shift<float>(long long, int, void *, void *, int, cudaStream_t);
 template cudaError_t run_tele_shift<double>(long long, int, void *, void *, int, cudaStream_t);
 
+template <typename F, bool PRE, int CL>
+static cudaError_t launch_tele2d_cl(int n_r, int n_d, double r_min, double dr, double dd, const void *s_r,
+                                    const double *r_src, int n_ev, double tol, int max_iter, void *tau,
+                                    void *pre, void *T, int *iters, cudaStream_t st) {
+    cudaLaunchConfig_t c = {};
+    c.gridDim = dim3((unsigned)n_ev * CL);
+    c.blockDim = dim3(kTeleThreads / (CL > 4 ? 4 : CL));
+    c.stream = st;
+    cudaLaunchAttribute at;
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = CL;
+    at.val.clusterDim.y = at.val.clusterDim.z = 1;
+    c.attrs = &at;
+    c.numAttrs = CL > 1 ? 1 : 0;
+    return cudaLaunchKernelEx(&c, tele2d_kernel<F, PRE, CL>, n_r, n_d, (F)r_min, (F)dr, (F)dd, (const F *)s_r,
+                              r_src, (F)tol, max_iter, (F *)tau, (Vec4<F> *)pre, (F *)T, iters);
+}
+
+template <typename F, bool PRE>
+static cudaError_t launch_tele2d(int cl, int n_r, int n_d, double r_min, double dr, double dd, const void *s_r,
+                                 const double *r_src, int n_ev, double tol, int max_iter, void *tau,
+                                 void *pre, void *T, int *iters, cudaStream_t st) {
+#define TTGB_TELE_CL(CL)                                                                               \
+    return launch_tele2d_cl<F, PRE, CL>(n_r, n_d, r_min, dr, dd, s_r, r_src, n_ev, tol, max_iter, tau, \
+                                        pre, T, iters, st)
+    if (cl == 8) TTGB_TELE_CL(8);
+    if (cl == 4) TTGB_TELE_CL(4);
+    if (cl == 2) TTGB_TELE_CL(2);
+    TTGB_TELE_CL(1);
+#undef TTGB_TELE_CL
+}
+
 template <typename F>
 cudaError_t run_tele2d(int n_r, int n_d, double r_min, double dr, double dd, const void *s_r,
                        const double *r_src, int n_ev, double tol, int max_iter, void *tau,
-                       void *T, int *iters, cudaStream_t st) {
-    tele2d_kernel<F><<<n_ev, kTeleThreads, 0, st>>>(n_r, n_d, (F)r_min, (F)dr, (F)dd,
-                                                    (const F *)s_r, r_src, (F)tol, max_iter,
-                                                    (F *)tau, (F *)T, iters);
+                       void *pre, void *T, int *iters, int n_sm, cudaStream_t st) {
+    // as many blocks an event as the SMs have room for
+    const int cl = 8 * n_ev <= n_sm ? 8 : 4 * n_ev <= n_sm ? 4 : 2 * n_ev <= n_sm ? 2 : 1;
+    cudaError_t e = pre ? launch_tele2d<F, true>(cl, n_r, n_d, r_min, dr, dd, s_r, r_src, n_ev, tol, max_iter, tau, pre, T, iters, st)
+                        : launch_tele2d<F, false>(cl, n_r, n_d, r_min, dr, dd, s_r, r_src, n_ev, tol, max_iter, tau, pre, T, iters, st);
+    if (e != cudaSuccess) return e;
     return cudaGetLastError();
 }
 
@@ -267,10 +336,10 @@ cudaError_t run_region_times(const GridC &g, int n_r, int n_d, double r_min, dou
 }
 
 template cudaError_t run_tele2d<float>(int, int, double, double, double, const void *,
-                                       const double *, int, double, int, void *, void *, int *,
+                                       const double *, int, double, int, void *, void *, void *, int *, int,
                                        cudaStream_t);
 template cudaError_t run_tele2d<double>(int, int, double, double, double, const void *,
-                                        const double *, int, double, int, void *, void *, int *,
+                                        const double *, int, double, int, void *, void *, void *, int *, int,
                                         cudaStream_t);
 template cudaError_t run_region_times<float>(const GridC &, int, int, double, double, double,
                                              const void *, int, const double *, void *,

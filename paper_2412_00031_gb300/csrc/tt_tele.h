@@ -7,12 +7,14 @@
 
 namespace ttgb {
 
-// 2-D traveltimes of n_ev events (one block each) on r = r_min + i dr, Delta = j dd:
-// s_r [n_r] of F, r_src [n_ev] double, tau scratch and T [n_ev][n_r][n_d] of F, iters [n_ev].
+// 2-D traveltimes of n_ev events (a block or a cluster of blocks each) on r = r_min + i dr,
+// Delta = j dd: s_r [n_r] of F, r_src [n_ev] double, tau scratch and T [n_ev][n_r][n_d] of F,
+// iters [n_ev]; pre: scratch of four F per node and event for the nodes' constants, or NULL
+// (computed at every update).
 template <typename F>
 cudaError_t run_tele2d(int n_r, int n_d, double r_min, double dr, double dd, const void *s_r,
                        const double *r_src, int n_ev, double tol, int max_iter, void *tau,
-                       void *T, int *iters, cudaStream_t st);
+                       void *pre, void *T, int *iters, int n_sm, cudaStream_t st);
 // The 2-D times interpolated at every node of the region: T [N][n_ev] of F; ev_ll [n_ev][2]
 // the events' latitude and longitude in radians.
 template <typename F>

@@ -120,14 +120,15 @@ typedef struct {
     long long spin_limit_ns;/* bound on every device-side wait; 0 = 2 s */
     int launch_blocks;      /* persistent sweep launch: 0 = automatic, else at most this many
                                blocks (results do not depend on it) */
-    int sweep_schedule;     /* forward sweep schedule: 0 = automatic; 1 = node hyperplanes;
+    int sweep_schedule;     /* forward sweep schedule: 0 = automatic; 1 = node hyperplanes
+                               (the planes of up to three orderings in flight together);
                                2, 3, 4 = tile hyperplanes with 2x4x8, 4x4x4, 2x8x8 tiles
                                (r x theta x phi). Results do not depend on it. */
     int adj_chunk;          /* adjoint: sources per launch (the slices run one after another);
                                0 = all sources in one launch. A launch runs its sources as up
                                to 4 barrier groups side by side. Results do not depend on it. */
     int fwd_groups;         /* node-hyperplane forward sweep: barrier groups per launch
-                               (1..8), 0 = automatic. Results do not depend on it. */
+                               (1..8), 0 = automatic (one). Results do not depend on it. */
     int fwd_slots;          /* forward sweep: 0 = every source of the call resident at once;
                                S > 0 (rounded up to a multiple of 32, below n_src) = retire and
                                refill: one launch keeps S sources in flight and a source that

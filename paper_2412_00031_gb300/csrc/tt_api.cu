@@ -71,6 +71,7 @@ struct tt_ctx {
     // teleseismic events: 2-D tau scratch, event radii / coordinates and iteration counts, the
     // 2-D nodes' constants
     DevBuf tele_tau, tele_aux, tele_pre;
+    DevBuf fwd_moved;  // the plane sweep's convergence flags
     int mg_key[4] = {0, 0, 0, 0};
     struct Tuned { int n_src, dtype, scheme, schedule, groups; };
     std::vector<Tuned> tuned;
@@ -163,22 +164,33 @@ tt_status build_schedule(tt_ctx *ctx, Schedule &S, int lo) {
     S.nb = g.nt - 2 * lo;
     S.nc = g.np - 2 * lo;
     S.n_planes = S.na + S.nb + S.nc - 2;
-    std::vector<unsigned int> nodes;
-    nodes.reserve((size_t)S.na * S.nb * S.nc);
+    // nodes of every plane in the order of (a, b); counted first, so that each goes straight to
+    // its place
     std::vector<int> off(S.n_planes + 1, 0);
-    for (int L = 0; L < S.n_planes; ++L) {
-        off[L] = (int)nodes.size();
-        for (int a = 0; a < S.na; ++a) {
-            if (a > L) break;
-            for (int b = 0; b < S.nb; ++b) {
-                int c = L - a - b;
-                if (c < 0) break;
-                if (c >= S.nc) continue;
-                nodes.push_back(((unsigned)a << 20) | ((unsigned)b << 10) | (unsigned)c);
-            }
+    for (int a = 0; a < S.na; ++a)
+        for (int b = 0; b < S.nb; ++b) {   // planes a + b .. a + b + nc - 1 gain a node
+            ++off[a + b];
+            if (a + b + S.nc < S.n_planes) --off[a + b + S.nc];
         }
+    for (int L = 1; L < S.n_planes; ++L) off[L] += off[L - 1];
+    for (int L = 0, sum = 0; L <= S.n_planes; ++L) {
+        const int n = L < S.n_planes ? off[L] : 0;
+        off[L] = sum;
+        sum += n;
     }
-    off[S.n_planes] = (int)nodes.size();
+    std::vector<unsigned int> nodes((size_t)off[S.n_planes]);
+    std::vector<int> at(off.begin(), off.end());
+    for (int a = 0; a < S.na; ++a)
+        for (int b = 0; b < S.nb; ++b) {
+            // bit 30 of the interior schedule: the second or last layer along an axis (whose
+            // updates complete a face's two layers)
+            const unsigned row = ((unsigned)a << 20) | ((unsigned)b << 10);
+            const unsigned edge = lo > 0 ? 1u << 30 : 0u;
+            const bool all = a == 1 || a == S.na - 1 || b == 1 || b == S.nb - 1;
+            int *q = at.data() + a + b;
+            for (int c = 0; c < S.nc; ++c)
+                nodes[q[c]++] = row | (unsigned)c | (all || c == 1 || c == S.nc - 1 ? edge : 0u);
+        }
     CK(cudaMalloc((void **)&S.nodes, nodes.size() * sizeof(unsigned int)));
     CK(cudaMalloc((void **)&S.off, off.size() * sizeof(int)));
     CK(cudaMemcpy(S.nodes, nodes.data(), nodes.size() * sizeof(unsigned int),
@@ -291,12 +303,11 @@ template <typename F> void free_geo(GeoTab<F> &t) {
 // Launch shape of a persistent sweep: as many co-resident blocks as useful (at most two per
 // SM), never more threads than the widest hyperplane needs.
 template <typename F>
-tt_status sweep_shape(tt_ctx *ctx, bool fwd, int B, const Schedule &S, int cap, int &grid,
-                      int &block, int &slots) {
+tt_status sweep_shape(tt_ctx *ctx, int B, const Schedule &S, int cap, int &grid, int &block,
+                      int &slots) {
     block = sizeof(F) == 4 ? 512 : 256;
-    size_t smem = (size_t)B * sizeof(F) * (fwd ? 1 : 2);
-    int per_sm = fwd ? forward_blocks_per_sm<F>(block, smem, false)
-                     : adjoint_blocks_per_sm<F>(block, smem);
+    size_t smem = (size_t)B * sizeof(F) * 2;
+    int per_sm = adjoint_blocks_per_sm<F>(block, smem);
     if (per_sm <= 0) return fail(ctx, TT_ECUDA, "sweep kernel cannot be resident (B = %d)", B);
     if (per_sm > 2) per_sm = 2;
     long long max_grid = (long long)per_sm * ctx->n_sm;
@@ -372,6 +383,7 @@ template <typename F> struct Work {
     Vec4<F> *t0c = nullptr, *coef = nullptr;
     F *partial = nullptr;
     int *conv_f = nullptr, *iters_f = nullptr, *conv_a = nullptr, *iters_a = nullptr;
+    int *moved = nullptr;                   // convergence flags of the plane sweep, 3 per source
     int *nact = nullptr, *flags = nullptr;  // flags: model, data index, receiver position
     BarrierState *bar = nullptr;
     long long *cq = nullptr;
@@ -445,6 +457,8 @@ template <typename F> tt_status work_from_ctx(tt_ctx *ctx, Work<F> &W, int B, in
     ENSURE(ctx->nact, sizeof(int) * kMaxBarrierGroups);
     ENSURE(ctx->bar, sizeof(BarrierState) * kMaxBarrierGroups);
     ENSURE(ctx->flags, kFlagInts * sizeof(int));
+    ENSURE(ctx->fwd_moved, sizeof(int) * 3 * (size_t)B);
+    W.moved = (int *)ctx->fwd_moved.p;
     W.src = (SrcC *)ctx->src.p;
     W.tabT = (Vec2<F> *)ctx->tabT.p;
     W.tabP = (Vec2<F> *)ctx->tabP.p;
@@ -705,8 +719,7 @@ tt_status enq_forward(tt_ctx *ctx, Work<F> &W, const tt_model *m, int B, void *d
         a.src_n = S;
         a.idx32 = (unsigned long long)g.N * (unsigned long long)(S > 8 ? S : 8) < (1ull << 32);
         const int block = 256;
-        int per_sm = forward_blocks_per_sm<F>(block, fwd_smem_bytes<F>(S, block), a.idx32 != 0,
-                                              a.scheme);
+        int per_sm = refill_blocks_per_sm<F>(block, refill_smem_bytes<F>(S), a.idx32 != 0, a.scheme);
         if (per_sm <= 0) return fail(ctx, TT_ECUDA, "sweep kernel cannot be resident");
         if (per_sm > kMaxBarrierGroups) per_sm = kMaxBarrierGroups;
         int max_grid = per_sm * ctx->n_sm;
@@ -726,7 +739,7 @@ tt_status enq_forward(tt_ctx *ctx, Work<F> &W, const tt_model *m, int B, void *d
         a.grp_blocks = gblocks;
         a.grp_src = gsrc;
         CK(launch_refill_setup<F>(a, ctx->st));
-        CK(launch_forward<F>(a, gblocks * groups, block, ctx->st));
+        CK(launch_refill<F>(a, gblocks * groups, block, ctx->st));
         ctx->stats[TT_STATS_FORWARD].block_threads = block;
         ctx->launches += 2;
         max_grid_used = gblocks * groups;
@@ -736,37 +749,15 @@ tt_status enq_forward(tt_ctx *ctx, Work<F> &W, const tt_model *m, int B, void *d
         a.src_lo = s0;
         a.src_n = n;
         int grid = 0;
-        if (sched == 1 || n < 32) {  // a tile task stages 32 sources: short slices use nodes
-            // 256-thread blocks; one barrier group per resident block slot of an SM, so
-            // each SM interleaves the groups; each group gets a multiple of 32 sources.
-            const int block = 256;
-            int per_sm = forward_blocks_per_sm<F>(block, fwd_smem_bytes<F>(n, block), a.idx32 != 0,
-                                                  a.scheme);
-            if (per_sm <= 0) return fail(ctx, TT_ECUDA, "sweep kernel cannot be resident");
-            if (per_sm > kMaxBarrierGroups) per_sm = kMaxBarrierGroups;
-            int max_grid = per_sm * ctx->n_sm;
-            if (o->launch_blocks > 0 && o->launch_blocks < max_grid) max_grid = o->launch_blocks;
-            const int wsrc = 32 * kFwdSourcesPerLane;  // sources of one warp
-            int groups = o->fwd_groups > 0 ? o->fwd_groups : per_sm;
-            if (groups > kMaxBarrierGroups) groups = kMaxBarrierGroups;
-            if (groups > (n + wsrc - 1) / wsrc) groups = (n + wsrc - 1) / wsrc;
-            if (groups > max_grid) groups = max_grid;
-            int gsrc = ((n + groups - 1) / groups + wsrc - 1) / wsrc * wsrc;
-            groups = (n + gsrc - 1) / gsrc;
-            int gblocks = max_grid / groups;
-            if ((long long)gblocks * block < gsrc) {
-                int need = (gsrc + block - 1) / block;
-                if ((long long)need * groups > (long long)per_sm * ctx->n_sm)
-                    return fail(ctx, TT_EINVAL, "slice of %d sources exceeds one resident launch", n);
-                gblocks = need;
-            }
-            grid = gblocks * groups;
-            a.n_bgroups = groups;
-            a.grp_blocks = gblocks;
-            a.grp_src = gsrc;
-            CK(launch_t0_cache<F>(a, ctx->st));
-            CK(launch_forward<F>(a, grid, block, ctx->st));
+        if (sched == 1 || n < 32) {  // a tile task stages 32 sources: short slices use planes
+            int block = 0, kernels = 0;
+            const cudaError_t e = run_plane_forward<F>(a, o->fwd_groups, W.moved, ctx->n_sm,
+                                                       o->launch_blocks, &grid, &block, &kernels, ctx->st);
+            if (e == cudaErrorInvalidConfiguration)
+                return fail(ctx, TT_EINVAL, "slice of %d sources exceeds one resident launch", n);
+            CK(e);
             ctx->stats[TT_STATS_FORWARD].block_threads = block;
+            ctx->launches += kernels;
         } else {
             int per_sm = forward_tiled_blocks_per_sm<F>(sched - 2, B);
             if (per_sm <= 0) return fail(ctx, TT_ECUDA, "tiled sweep cannot be resident");
@@ -791,8 +782,8 @@ tt_status enq_forward(tt_ctx *ctx, Work<F> &W, const tt_model *m, int B, void *d
             CK(launch_t0_cache<F>(a, ctx->st));
             CK(launch_forward_tiled<F>(map_tau, map_rec, map_t0c, a, sched - 2, grid, ctx->st));
             ctx->stats[TT_STATS_FORWARD].block_threads = kTileThreads;
+            ctx->launches += 2;
         }
-        ctx->launches += 2;
         if (grid > max_grid_used) max_grid_used = grid;
     }
     CK(record(ctx, ctx->ev_stop[TT_STATS_FORWARD]));
@@ -901,8 +892,7 @@ tt_status enq_adjoint(tt_ctx *ctx, Work<F> &W, const tt_model *m, int B, const v
         }
         grid = grp_blocks * groups;
         slots = 0;
-    } else if ((s = sweep_shape<F>(ctx, false, B, ctx->full, o->launch_blocks, grid, block,
-                                   slots)) != TT_OK) {
+    } else if ((s = sweep_shape<F>(ctx, B, ctx->full, o->launch_blocks, grid, block, slots)) != TT_OK) {
         return s;
     }
     const GeoTab<F> &t = geo<F>(ctx);
@@ -1304,7 +1294,7 @@ void tt_ctx_destroy(tt_ctx *ctx) {
                       &ctx->tele_tau, &ctx->tele_aux, &ctx->tele_pre, &ctx->net_img, &ctx->net_timg,
                       &ctx->net_rows, &ctx->ord_perm, &ctx->ord_pts, &ctx->ord_src,
                       &ctx->ord_tabT, &ctx->ord_tabP, &ctx->ord_tau, &ctx->ord_iters,
-                      &ctx->ord_conv};
+                      &ctx->ord_conv, &ctx->fwd_moved};
     for (DevBuf *b : bufs)
         if (b->p) cudaFree(b->p);
     if (ctx->h_loss) cudaFreeHost(ctx->h_loss);
@@ -1656,10 +1646,9 @@ tt_status forward_tele_impl(tt_ctx *ctx, const tt_model *m, int n_ev, void *d_T,
                             const tt_opts *o, int *h_iters) {
     const GridC &g = ctx->g;
     ENSURE(ctx->rec, sizeof(NodeRec<F>) * (size_t)g.N);
-    ENSURE(ctx->partial, partial_bytes(ctx, n_ev, sizeof(F)));
     ENSURE(ctx->conv, sizeof(int) * (size_t)n_ev);
     ENSURE(ctx->iters, sizeof(int) * (size_t)n_ev);
-    ENSURE(ctx->nact, sizeof(int) * kMaxBarrierGroups);
+    ENSURE(ctx->fwd_moved, sizeof(int) * 3 * (size_t)n_ev);
     ENSURE(ctx->bar, sizeof(BarrierState) * kMaxBarrierGroups);
     ENSURE(ctx->flags, kFlagInts * sizeof(int));
     NodeRec<F> *rec = (NodeRec<F> *)ctx->rec.p;
@@ -1667,7 +1656,6 @@ tt_status forward_tele_impl(tt_ctx *ctx, const tt_model *m, int n_ev, void *d_T,
     BarrierState *bar = (BarrierState *)ctx->bar.p;
     CK(cudaMemsetAsync(conv, 0, sizeof(int) * (size_t)n_ev, ctx->st));
     CK(cudaMemsetAsync(iters, 0, sizeof(int) * (size_t)n_ev, ctx->st));
-    CK(cudaMemsetAsync(ctx->nact.p, 0, sizeof(int) * kMaxBarrierGroups, ctx->st));
     CK(cudaMemsetAsync(bar, 0, sizeof(BarrierState) * kMaxBarrierGroups, ctx->st));
     CK(cudaMemsetAsync(flags, 0, 4 * sizeof(int), ctx->st));
     CK(run_node_records<F>(g, m->d_s, m->d_xi, m->d_eta, ctx->gd.h2, ctx->gd.cost, rec, flags,
@@ -1679,6 +1667,9 @@ tt_status forward_tele_impl(tt_ctx *ctx, const tt_model *m, int n_ev, void *d_T,
     a.g = g;
     a.B = n_ev;
     a.scheme = 3;
+    a.na = g.nr - 2;
+    a.nb = g.nt - 2;
+    a.nc = g.np - 2;
     a.n_planes = ctx->interior.n_planes;
     a.er = (F)(0.5 / g.dr);
     a.rec = rec;
@@ -1686,42 +1677,20 @@ tt_status forward_tele_impl(tt_ctx *ctx, const tt_model *m, int n_ev, void *d_T,
     a.nodes = ctx->interior.nodes;
     a.off = ctx->interior.off;
     a.bar = bar;
-    a.partial = (F *)ctx->partial.p;
     a.conv = conv;
     a.iters = iters;
-    a.n_active = (int *)ctx->nact.p;
     a.tol = (F)o->tol_fwd;
     a.max_iter = o->max_iter_fwd;
     a.spin_ns = spin_ns(o);
     a.src_lo = 0;
     a.src_n = n_ev;
-    a.idx32 = (unsigned long long)g.N * (unsigned long long)(n_ev > 8 ? n_ev : 8) < (1ull << 32);
-    // 256-thread blocks, one barrier group per resident block slot of an SM (as the
-    // forward sweep), each group a multiple of one warp's sources
-    const int block = 256;
-    int per_sm = forward_blocks_per_sm<F>(block, fwd_smem_bytes<F>(n_ev, block), a.idx32 != 0, 3);
-    if (per_sm <= 0) return fail(ctx, TT_ECUDA, "teleseismic sweep cannot be resident");
-    if (per_sm > kMaxBarrierGroups) per_sm = kMaxBarrierGroups;
-    int max_grid = per_sm * ctx->n_sm;
-    if (o->launch_blocks > 0 && o->launch_blocks < max_grid) max_grid = o->launch_blocks;
-    const int wsrc = 32 * kFwdSourcesPerLane;
-    int groups = o->fwd_groups > 0 ? o->fwd_groups : per_sm;
-    if (groups > (n_ev + wsrc - 1) / wsrc) groups = (n_ev + wsrc - 1) / wsrc;
-    if (groups > max_grid) groups = max_grid;
-    int gsrc = ((n_ev + groups - 1) / groups + wsrc - 1) / wsrc * wsrc;
-    groups = (n_ev + gsrc - 1) / gsrc;
-    int gblocks = max_grid / groups;
-    if ((long long)gblocks * block < gsrc) {
-        const int need = (gsrc + block - 1) / block;
-        if ((long long)need * groups > (long long)per_sm * ctx->n_sm)
-            return fail(ctx, TT_EINVAL, "%d events exceed one resident launch", n_ev);
-        gblocks = need;
-    }
-    a.n_bgroups = groups;
-    a.grp_blocks = gblocks;
-    a.grp_src = gsrc;
+    int grid = 0, block = 0, kernels = 0;
     CK(record(ctx, ctx->ev_start[TT_STATS_FORWARD]));
-    CK(launch_forward<F>(a, gblocks * groups, block, ctx->st));
+    const cudaError_t le = run_plane_forward<F>(a, o->fwd_groups, (int *)ctx->fwd_moved.p, ctx->n_sm,
+                                                o->launch_blocks, &grid, &block, &kernels, ctx->st);
+    if (le == cudaErrorInvalidConfiguration)
+        return fail(ctx, TT_EINVAL, "%d events exceed one resident launch", n_ev);
+    CK(le);
     CK(record(ctx, ctx->ev_stop[TT_STATS_FORWARD]));
     CK(run_tele_shift<F>(g.N, n_ev, d_T, ctx->tele_aux.p, 1, ctx->st));
     ctx->launches += 5;
@@ -1760,7 +1729,7 @@ tt_status forward_tele_impl(tt_ctx *ctx, const tt_model *m, int n_ev, void *d_T,
     S.node_updates = upd;
     S.node_sweeps = 8LL * imax * inner;
     S.iters_max = imax;
-    S.grid_blocks = gblocks * groups;
+    S.grid_blocks = grid;
     S.block_threads = block;
     if (left)
         return fail(ctx, TT_ENOTCONVERGED,
@@ -2420,6 +2389,7 @@ template <typename F> tt_status plan_alloc(tt_plan *p, Work<F> &W) {
     TTGB_GET(conv_a, sizeof(int) * B);
     TTGB_GET(iters_a, sizeof(int) * B);
     TTGB_GET(nact, sizeof(int) * kMaxBarrierGroups);
+    TTGB_GET(moved, sizeof(int) * 3 * (size_t)B);
     TTGB_GET(flags, kFlagInts * sizeof(int));
     TTGB_GET(bar, sizeof(BarrierState) * kMaxBarrierGroups);
     TTGB_GET(cq, sizeof(long long) * S);

@@ -468,41 +468,50 @@ __device__ __forceinline__ void barrier_begin() {
     if (threadIdx.x == 0) s_bar_target = 0;
 }
 
-// Returns false when the barrier (or an earlier one in another block) timed out. nblocks is
-// the number of blocks that take part (all blocks of the launch, or one barrier group).
+// One thread of each block posts the block's arrival. release: the fence orders the block's writes
+// (made visible to this thread by a block barrier) before the arrival; the acquiring load of
+// the wait pairs with the other blocks' fences, and a block barrier passes the ordering on.
+// nblocks is the number of blocks that take part (all blocks of the launch, or one group).
+__device__ __forceinline__ void barrier_post(BarrierState *bs, unsigned int nblocks) {
+    s_bar_target += nblocks;
+    fence_acq_rel_gpu();
+    red_relaxed_add(&bs->arrived, 1ull);
+}
+
+// The same thread's wait: 0 when the barrier (or an earlier one in another block) timed out.
+__device__ __forceinline__ int barrier_poll(BarrierState *bs, unsigned long long limit_ns) {
+    int good = 1;
+    const unsigned long long target = s_bar_target;
+    // another block's timeout, read together with the first poll rather than after the
+    // wait, so that it adds no round trip to the barrier (a timeout during this wait is
+    // then seen at the next barrier, which the block that timed out never reaches)
+    const int st0 = ld_status(&bs->status);
+    if (ld_acquire(&bs->arrived) < target) {
+        if (st0 != 0) good = 0;  // a block gave up earlier: no one waits for it
+        const unsigned long long t0 = global_ns();
+        unsigned int ns = 16;
+        while (good && ld_acquire(&bs->arrived) < target) {
+            if (global_ns() - t0 > limit_ns) {
+                atomicExch(&bs->status, (int)kDevTimeout);
+                good = 0;
+                break;
+            }
+            __nanosleep(ns);
+            if (ns < 64) ns <<= 1;
+        }
+    }
+    if (good && st0 != 0) good = 0;
+    return good;
+}
+
+// All threads of the block; false when the barrier (or an earlier one in another block) timed out.
 __device__ __forceinline__ bool grid_barrier(BarrierState *bs, unsigned long long limit_ns,
                                              unsigned int nblocks) {
     __shared__ int ok;
     __syncthreads();
     if (threadIdx.x == 0) {
-        int good = 1;
-        const unsigned long long target = s_bar_target + nblocks;
-        s_bar_target = target;
-        // release: the fence orders the block's writes (made visible to this thread by
-        // __syncthreads) before the arrival; the acquiring load below pairs with the other
-        // blocks' fences, and __syncthreads passes the ordering on to the whole block
-        fence_acq_rel_gpu();
-        red_relaxed_add(&bs->arrived, 1ull);
-        // another block's timeout, read together with the first poll rather than after the
-        // wait, so that it adds no round trip to the barrier (a timeout during this wait is
-        // then seen at the next barrier, which the block that timed out never reaches)
-        const int st0 = ld_status(&bs->status);
-        if (ld_acquire(&bs->arrived) < target) {
-            if (st0 != 0) good = 0;  // a block gave up earlier: no one waits for it
-            const unsigned long long t0 = global_ns();
-            unsigned int ns = 16;
-            while (good && ld_acquire(&bs->arrived) < target) {
-                if (global_ns() - t0 > limit_ns) {
-                    atomicExch(&bs->status, (int)kDevTimeout);
-                    good = 0;
-                    break;
-                }
-                __nanosleep(ns);
-                if (ns < 64) ns <<= 1;
-            }
-        }
-        if (good && st0 != 0) good = 0;
-        ok = good;
+        barrier_post(bs, nblocks);
+        ok = barrier_poll(bs, limit_ns);
     }
     __syncthreads();
     return ok != 0;

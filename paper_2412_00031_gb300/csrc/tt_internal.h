@@ -105,19 +105,29 @@ template <typename F> struct AdjArgs {
     unsigned long long spin_ns;
 };
 
-// Dynamic shared memory of the node-hyperplane forward sweep: the per-source maxima of a
-// barrier group, then (staged kernel) the two-stage copy buffers of every thread.
-template <typename F> __host__ __device__ inline size_t fwd_err_bytes(int grp_src) {
+// Dynamic shared memory of the retire-and-refill sweep: the per-source maxima of a barrier group.
+template <typename F> inline size_t refill_smem_bytes(int grp_src) {
     return ((size_t)grp_src * sizeof(F) + 127) / 128 * 128;
 }
-template <typename F> size_t fwd_smem_bytes(int grp_src, int block);
 
 // Launchers (tt_sweep.cu). They return a cudaError_t of the launch itself.
-template <typename F> cudaError_t launch_forward(const FwdArgs<F> &a, int grid, int block,
-                                                 cudaStream_t st);
+template <typename F> cudaError_t launch_refill(const FwdArgs<F> &a, int grid, int block,
+                                                cudaStream_t st);
 template <typename F> cudaError_t launch_adjoint(const AdjArgs<F> &a, int grid, int block,
                                                  cudaStream_t st);
-template <typename F> int forward_blocks_per_sm(int block, size_t smem, bool idx32, int scheme = 0);
+// Plane-by-plane sweeps (tt_plane.cu): barrier groups of grp_src sources and grp_blocks blocks;
+// ordering o of an iteration begins at time step start[o].
+struct PlaneShape {
+    int grp_src, grp_blocks;
+    int start[8], steps;
+    int *moved;          // [3][src_n], by iteration mod 3: the source has not converged
+};
+// The sources [src_lo, src_lo + src_n) of a; groups: barrier groups (0 = 1); moved: 3 * src_n ints.
+// grid, block and kernels receive the launch's shape and the number of kernels launched.
+template <typename F>
+cudaError_t run_plane_forward(FwdArgs<F> a, int groups, int *moved, int n_sm, int launch_blocks, int *grid,
+                              int *block, int *kernels, cudaStream_t st);
+template <typename F> int refill_blocks_per_sm(int block, size_t smem, bool idx32, int scheme);
 template <typename F> cudaError_t launch_t0_cache(const FwdArgs<F> &a, cudaStream_t st);
 // Slot table of the retire-and-refill mode: slot s < n_slots takes source s.
 template <typename F> cudaError_t launch_refill_setup(const FwdArgs<F> &a, cudaStream_t st);
@@ -135,7 +145,7 @@ cudaError_t launch_forward_tiled(const CUtensorMap &map_tau, const CUtensorMap &
                                  int grid, cudaStream_t st);
 template <typename F> int forward_tiled_blocks_per_sm(int shape, int B);
 constexpr int kTileThreads = 256;
-// Sources one lane of the node-hyperplane forward sweep updates at each node (a warp covers
+// Sources one lane of the retire-and-refill sweep updates at each node (a warp covers
 // 32 x this many consecutive sources); barrier groups are sized in multiples of a warp's.
 #ifndef TTGB_FWD_NS
 #define TTGB_FWD_NS 2

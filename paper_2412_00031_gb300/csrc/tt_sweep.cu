@@ -11,10 +11,9 @@
 #include <cuda_runtime.h>
 
 #include "tt_internal.h"
+#include "tt_update.cuh"
 
 namespace ttgb {
-
-template <typename F> __device__ __forceinline__ F fmax_(F a, F b) { return a > b ? a : b; }
 
 __device__ __forceinline__ void atomic_max_nonneg(float *p, float v) {
     atomicMax(reinterpret_cast<unsigned int *>(p), __float_as_uint(v));
@@ -29,7 +28,7 @@ __device__ __forceinline__ unsigned smem_u32(const void *p) {
 }
 
 __device__ __forceinline__ void unpack(unsigned int pk, int &a, int &b, int &c) {
-    a = (int)(pk >> 20);
+    a = (int)(pk >> 20) & 1023;   // bit 30 is a flag of the interior schedule
     b = (int)((pk >> 10) & 1023u);
     c = (int)(pk & 1023u);
 }
@@ -194,18 +193,15 @@ template <typename F> __global__ void refill_setup_kernel(FwdArgs<F> a) {
     if (has) a.slot_srcc[x] = a.src_all[x];
 }
 
-// Node-hyperplane schedule. The launch is split into barrier groups: group g owns a
-// contiguous slice of the launch's sources and a contiguous range of blocks, runs the whole
-// solve of its slice with its own grid barrier and convergence test, and so never waits for
-// another group; on each SM the warps of one group keep issuing while another group's warps
-// wait at their barrier.
+// Retire-and-refill sweep (opts.fwd_slots), hyperplane by hyperplane. The launch is split into
+// barrier groups: group g owns a contiguous slice of the launch's slots and a contiguous range of
+// blocks, and runs with its own grid barrier and convergence test.
 //
-// Within a group, a warp covers 64 consecutive sources of one node: lane l holds sources
-// l and l + 32 of its 64, so both of a lane's accesses are coalesced 128-byte lines and the
-// second is the first plus a constant offset. A slot is the set of warps that cover the
-// group's sources (padded to whole warps); on a hyperplane each slot takes the nodes slot,
-// slot + slots, ... The schedule is static, so the index of a thread's next node, the
-// bounds of the next hyperplane and the index of its first node there are read one step
+// Within a group, a warp covers 64 consecutive source slots of one node: lane l holds l and
+// l + 32 of its 64, so both of a lane's accesses are coalesced 128-byte lines. A node slot is the
+// set of warps that cover the group's sources (padded to whole warps); on a hyperplane each takes
+// the nodes slot, slot + slots, ... The schedule is static, so the index of a thread's next node,
+// the bounds of the next hyperplane and the index of its first node there are read one step
 // ahead (the latter two before the barrier), off the critical path. The node record (8
 // values shared by the warp) is read by every lane as two broadcast 16-byte loads. The
 // factor cache is read once per sweep and streamed past L2 (evict-first), so that it does
@@ -256,38 +252,25 @@ __device__ __forceinline__ Vec4<double> ld_stream(const Vec4<double> *p) {
     return Vec4<double>{v0.x, v0.y, v1.x, v1.y};
 }
 
-// Lax-Friedrichs update of one (node, source): tau at p, its six neighbours at p +- sr,
-// p +- st, p +- sp; c = the cached factors. Returns |change| (0 on the fixed set).
-__device__ __forceinline__ unsigned bits_of(float x) { return __float_as_uint(x); }
-__device__ __forceinline__ unsigned long long bits_of(double x) {
-    return (unsigned long long)__double_as_longlong(x);
-}
-
+// Update of one (node, source): tau at p, v its stencil (sweep_update), c the cached factors.
+// Returns |change| (0 on the fixed set).
 template <typename F, int SCHEME>
 __device__ __forceinline__ F update_one(F *p, const F *v, const Vec4<F> &c, const NodeRec<F> &R,
                                         F er) {
     if (!(c.x > (F)0)) return (F)0;
-    const F tn =
-        SCHEME == 2   ? godunov_aniso_core<F>(c.x, c.y, c.z, c.w, v[0], v[1], v[2], v[3], v[4], v[5], v[6], R, er)
-        : SCHEME == 1 ? godunov_core<F>(c.x, c.y, c.z, c.w, v[0], v[1], v[2], v[3], v[4], v[5], v[6], R, er)
-                      : lf_core<F>(c.x, c.y, c.z, c.w, v[0], v[1], v[2], v[3], v[4], v[5], v[6], R, er);
+    const F tn = sweep_update<F, SCHEME>(v, c, R, er);
     // a value that keeps its bits is not stored, so that its line is not made dirty (late
     // in a solve most values have stopped changing)
     if (bits_of(tn) != bits_of(v[0])) *p = tn;
     return fabs(tn - v[0]);
 }
 
-// I: index type of the [node][source] fields (32-bit when every index fits).
-// REFILL: the retire-and-refill mode (compiled separately, so that the resident launch
-// carries none of its code). SCHEME: the local solver, 0 Lax-Friedrichs (lf_core), 1 Godunov
-// (godunov_core, isotropic models), 2 Godunov for anisotropic models (godunov_aniso_core),
-// 3 Lax-Friedrichs on T itself with the faces held fixed (the region's solve of teleseismic
-// events: lf_core with T0 = 1 and no factor gradient, no factor cache read, no fixed set,
-// no face extrapolation; the "sources" are the events).
-template <typename F, typename I, bool REFILL, int SCHEME>
-__global__ void __launch_bounds__(256, (SCHEME == 0 || SCHEME == 3) ? TTGB_FWD_MIN_BLOCKS
-                                                                    : TTGB_GOD_MIN_BLOCKS)
-    fwd_sweep_kernel(FwdArgs<F> a) {
+// I: index type of the [node][source] fields (32-bit when every index fits). SCHEME: the local
+// solver, 0 Lax-Friedrichs (lf_core), 1 Godunov (godunov_core, isotropic models), 2 Godunov for
+// anisotropic models (godunov_aniso_core).
+template <typename F, typename I, int SCHEME>
+__global__ void __launch_bounds__(256, SCHEME == 0 ? TTGB_FWD_MIN_BLOCKS : TTGB_GOD_MIN_BLOCKS)
+    refill_sweep_kernel(FwdArgs<F> a) {
     constexpr int NS = kFwdSourcesPerLane;              // sources of one lane: l0 + 32 h
     extern __shared__ unsigned char smem_raw[];
     F *s_err = reinterpret_cast<F *>(smem_raw);
@@ -322,19 +305,16 @@ __global__ void __launch_bounds__(256, (SCHEME == 0 || SCHEME == 3) ? TTGB_FWD_M
     F *tau = a.tau;
 
     // retire-and-refill: load the group's first sources into their slots
-    if (REFILL) {
-        refill_slots<F>(a, src0, Bg, blk);
-        if (!grid_barrier(bar, a.spin_ns, nblk)) return;
-    }
-    // with refill a group runs until its queue is empty; each source still stops at max_iter
-    const long long it_end = REFILL ? (long long)a.max_iter * (a.n_all + 1) : a.max_iter;
+    refill_slots<F>(a, src0, Bg, blk);
+    if (!grid_barrier(bar, a.spin_ns, nblk)) return;
+    // a group runs until its queue is empty; each source still stops at max_iter
+    const long long it_end = (long long)a.max_iter * (a.n_all + 1);
     for (long long it = 0; it < it_end; ++it) {
         bool act[NS];
         bool any = false;
 #pragma unroll
         for (int h = 0; h < NS; ++h) {
-            act[h] = okh[h] && (REFILL ? ((volatile int *)a.slot_src)[b + 32 * h] >= 0
-                                       : ((volatile int *)a.conv)[b + 32 * h] == 0);
+            act[h] = okh[h] && ((volatile int *)a.slot_src)[b + 32 * h] >= 0;
             any = any || act[h];
         }
         const bool busy = lane_ok && __any_sync(0xffffffffu, any);  // uniform
@@ -374,8 +354,7 @@ __global__ void __launch_bounds__(256, (SCHEME == 0 || SCHEME == 3) ? TTGB_FWD_M
                             v[h][4] = ph[-ost];
                             v[h][5] = ph[osp];
                             v[h][6] = ph[-osp];
-                            c[h] = SCHEME == 3 ? Vec4<F>{(F)1, (F)0, (F)0, (F)0}
-                                               : ld_stream(pc + 32 * h);
+                            c[h] = ld_stream(pc + 32 * h);
                         }
                         const NodeRec<F> R = rec_vec(a.rec + n);
 #pragma unroll
@@ -392,11 +371,10 @@ __global__ void __launch_bounds__(256, (SCHEME == 0 || SCHEME == 3) ? TTGB_FWD_M
                 qa = qa_next;
                 qe = qe_next;
             }
-            if (SCHEME != 3)  // SCHEME 3 holds the faces fixed
-                for (int axis = 0; axis < 3; ++axis) {
-                    if (any) extrapolate_lane<F, NS>(a, b, act, axis, slot, slots);
-                    if (!grid_barrier(bar, a.spin_ns, nblk)) return;
-                }
+            for (int axis = 0; axis < 3; ++axis) {
+                if (any) extrapolate_lane<F, NS>(a, b, act, axis, slot, slots);
+                if (!grid_barrier(bar, a.spin_ns, nblk)) return;
+            }
         }
         // Per-source largest update of this iteration: block maximum, then a fixed-order
         // maximum over the group's blocks by its first block, which also decides convergence.
@@ -413,52 +391,40 @@ __global__ void __launch_bounds__(256, (SCHEME == 0 || SCHEME == 3) ? TTGB_FWD_M
             if (threadIdx.x == 0) s_cnt = 0;
             __syncthreads();
             for (int x = src0 + threadIdx.x; x < src0 + Bg; x += blockDim.x) {
-                if (REFILL) {
-                    // slots: a finished source hands its slot to the next queued source
-                    a.slot_fill[x] = 0;
-                    const int s = a.slot_src[x];
-                    if (s < 0) continue;
-                    F m = 0;
-                    for (int c = grp * a.grp_blocks; c < (grp + 1) * a.grp_blocks; ++c)
-                        m = fmax_(m, ((volatile F *)a.partial)[(long long)c * B + x]);
-                    const int its = a.slot_it[x] + 1;
-                    a.slot_it[x] = its;
-                    if (!(m < a.tol) && its < a.max_iter) {
-                        atomicAdd(&s_cnt, 1);
-                        continue;
-                    }
-                    a.iters[s] = its;
-                    a.conv[s] = m < a.tol ? 1 : 0;
-                    const int nw = atomicAdd(a.queue, 1);
-                    a.slot_prev[x] = s;
-                    a.slot_fill[x] = 1;
-                    a.slot_it[x] = 0;
-                    if (nw < a.n_all) {
-                        a.slot_src[x] = nw;
-                        a.slot_srcc[x] = a.src_all[nw];
-                        atomicAdd(&s_cnt, 1);
-                    } else {
-                        a.slot_src[x] = -1;
-                    }
-                    continue;
-                }
-                if (a.conv[x]) continue;
+                // slots: a finished source hands its slot to the next queued source
+                a.slot_fill[x] = 0;
+                const int s = a.slot_src[x];
+                if (s < 0) continue;
                 F m = 0;
                 for (int c = grp * a.grp_blocks; c < (grp + 1) * a.grp_blocks; ++c)
                     m = fmax_(m, ((volatile F *)a.partial)[(long long)c * B + x]);
-                a.iters[x] = (int)it + 1;
-                if (m < a.tol) a.conv[x] = 1;
-                else atomicAdd(&s_cnt, 1);
+                const int its = a.slot_it[x] + 1;
+                a.slot_it[x] = its;
+                if (!(m < a.tol) && its < a.max_iter) {
+                    atomicAdd(&s_cnt, 1);
+                    continue;
+                }
+                a.iters[s] = its;
+                a.conv[s] = m < a.tol ? 1 : 0;
+                const int nw = atomicAdd(a.queue, 1);
+                a.slot_prev[x] = s;
+                a.slot_fill[x] = 1;
+                a.slot_it[x] = 0;
+                if (nw < a.n_all) {
+                    a.slot_src[x] = nw;
+                    a.slot_srcc[x] = a.src_all[nw];
+                    atomicAdd(&s_cnt, 1);
+                } else {
+                    a.slot_src[x] = -1;
+                }
             }
             __syncthreads();
             if (threadIdx.x == 0) ((volatile int *)a.n_active)[grp] = s_cnt;
         }
         if (!grid_barrier(bar, a.spin_ns, nblk)) return;
-        if (REFILL) {
-            // retire the finished columns and load the new sources, then start them together
-            refill_slots<F>(a, src0, Bg, blk);
-            if (!grid_barrier(bar, a.spin_ns, nblk)) return;
-        }
+        // retire the finished columns and load the new sources, then start them together
+        refill_slots<F>(a, src0, Bg, blk);
+        if (!grid_barrier(bar, a.spin_ns, nblk)) return;
         if (((volatile int *)a.n_active)[grp] == 0) break;
     }
     barrier_end(bar, nblk);
@@ -1180,32 +1146,20 @@ __global__ void __launch_bounds__(256, TTGB_ADJ_MIN_BLOCKS) adj_face_kernel(AdjA
 
 // ------------------------------------------------------------------------ launchers
 
-// The node-hyperplane sweep kernel of one variant.
-template <typename F> void *fwd_kernel_ptr(bool refill, bool idx32, int scheme) {
-    if (scheme == 3)  // no refill mode
-        return idx32 ? (void *)fwd_sweep_kernel<F, unsigned, false, 3>
-                     : (void *)fwd_sweep_kernel<F, long long, false, 3>;
+// The retire-and-refill kernel of one variant.
+template <typename F> void *refill_kernel_ptr(bool idx32, int scheme) {
     if (scheme == 2)
-        return refill ? (idx32 ? (void *)fwd_sweep_kernel<F, unsigned, true, 2>
-                               : (void *)fwd_sweep_kernel<F, long long, true, 2>)
-                      : (idx32 ? (void *)fwd_sweep_kernel<F, unsigned, false, 2>
-                               : (void *)fwd_sweep_kernel<F, long long, false, 2>);
+        return idx32 ? (void *)refill_sweep_kernel<F, unsigned, 2> : (void *)refill_sweep_kernel<F, long long, 2>;
     if (scheme == 1)
-        return refill ? (idx32 ? (void *)fwd_sweep_kernel<F, unsigned, true, 1>
-                               : (void *)fwd_sweep_kernel<F, long long, true, 1>)
-                      : (idx32 ? (void *)fwd_sweep_kernel<F, unsigned, false, 1>
-                               : (void *)fwd_sweep_kernel<F, long long, false, 1>);
-    return refill ? (idx32 ? (void *)fwd_sweep_kernel<F, unsigned, true, 0>
-                           : (void *)fwd_sweep_kernel<F, long long, true, 0>)
-                  : (idx32 ? (void *)fwd_sweep_kernel<F, unsigned, false, 0>
-                           : (void *)fwd_sweep_kernel<F, long long, false, 0>);
+        return idx32 ? (void *)refill_sweep_kernel<F, unsigned, 1> : (void *)refill_sweep_kernel<F, long long, 1>;
+    return idx32 ? (void *)refill_sweep_kernel<F, unsigned, 0> : (void *)refill_sweep_kernel<F, long long, 0>;
 }
 
 template <typename F>
-cudaError_t launch_forward(const FwdArgs<F> &a, int grid, int block, cudaStream_t st) {
+cudaError_t launch_refill(const FwdArgs<F> &a, int grid, int block, cudaStream_t st) {
     void *args[] = {const_cast<FwdArgs<F> *>(&a)};
-    const size_t smem = fwd_smem_bytes<F>(a.grp_src, block);
-    void *fn = fwd_kernel_ptr<F>(a.refill != 0, a.idx32 != 0, a.scheme);
+    const size_t smem = refill_smem_bytes<F>(a.grp_src);
+    void *fn = refill_kernel_ptr<F>(a.idx32 != 0, a.scheme);
     cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     return cudaLaunchCooperativeKernel(fn, dim3(grid), dim3(block), args, smem, st);
@@ -1224,13 +1178,9 @@ template <typename F> cudaError_t launch_refill_setup(const FwdArgs<F> &a, cudaS
     return cudaGetLastError();
 }
 
-template <typename F> size_t fwd_smem_bytes(int grp_src, int) {
-    return fwd_err_bytes<F>(grp_src);
-}
-
-template <typename F> int forward_blocks_per_sm(int block, size_t smem, bool idx32, int scheme) {
+template <typename F> int refill_blocks_per_sm(int block, size_t smem, bool idx32, int scheme) {
     int n = 0;
-    void *fn = fwd_kernel_ptr<F>(false, idx32, scheme);
+    void *fn = refill_kernel_ptr<F>(idx32, scheme);
     if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
         cudaSuccess)
         return 0;
@@ -1347,14 +1297,12 @@ template cudaError_t launch_adjoint_faces<double>(const AdjArgs<double> &, int, 
 template int adjoint_faces_blocks_per_sm<float>(int, size_t);
 template int adjoint_faces_blocks_per_sm<double>(int, size_t);
 
-template cudaError_t launch_forward<float>(const FwdArgs<float> &, int, int, cudaStream_t);
-template cudaError_t launch_forward<double>(const FwdArgs<double> &, int, int, cudaStream_t);
+template cudaError_t launch_refill<float>(const FwdArgs<float> &, int, int, cudaStream_t);
+template cudaError_t launch_refill<double>(const FwdArgs<double> &, int, int, cudaStream_t);
 template cudaError_t launch_adjoint<float>(const AdjArgs<float> &, int, int, cudaStream_t);
 template cudaError_t launch_adjoint<double>(const AdjArgs<double> &, int, int, cudaStream_t);
-template size_t fwd_smem_bytes<float>(int, int);
-template size_t fwd_smem_bytes<double>(int, int);
-template int forward_blocks_per_sm<float>(int, size_t, bool, int);
-template int forward_blocks_per_sm<double>(int, size_t, bool, int);
+template int refill_blocks_per_sm<float>(int, size_t, bool, int);
+template int refill_blocks_per_sm<double>(int, size_t, bool, int);
 template int adjoint_blocks_per_sm<float>(int, size_t);
 template int adjoint_blocks_per_sm<double>(int, size_t);
 

@@ -22,7 +22,7 @@ cudaError_t run_region_times(const GridC &g, int n_r, int n_d, double r_min, dou
                              double dd, const void *T2, int n_ev, const double *ev_ll, void *T,
                              cudaStream_t st);
 
-// The region's solve itself is the node-hyperplane sweep (tt_sweep.cu) with SCHEME 3, on
+// The region's solve itself is the plane sweep (tt_plane.cu) with SCHEME 3, on
 // T - c_e: sign < 0 saves c_e = T[node 0][e] into c [n_ev] and subtracts it from every node of
 // event e; sign > 0 adds it back.
 template <typename F>

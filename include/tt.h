@@ -125,8 +125,7 @@ typedef struct {
                                2, 3, 4 = tile hyperplanes with 2x4x8, 4x4x4, 2x8x8 tiles
                                (r x theta x phi). Results do not depend on it. */
     int adj_chunk;          /* adjoint: sources per launch (the slices run one after another);
-                               0 = all sources in one launch. A launch runs its sources as up
-                               to 4 barrier groups side by side. Results do not depend on it. */
+                               0 = all sources in one launch. Results do not depend on it. */
     int fwd_groups;         /* node-hyperplane forward sweep: barrier groups per launch
                                (1..8), 0 = automatic (one). Results do not depend on it. */
     int fwd_slots;          /* forward sweep: 0 = every source of the call resident at once;
@@ -142,7 +141,7 @@ typedef struct {
                                M grad T, the Schur-complement form of M on each axis subset).
                                The Godunov solvers run on the node-hyperplane schedule. */
     int adj_groups;         /* adjoint: barrier groups per launch (1..8; each gets at least 32
-                               sources), 0 = automatic (one per 64 sources, at most 4).
+                               sources), 0 = automatic (one).
                                Results do not depend on it. */
     int fwd_order;          /* 0 = sweep a batch of 64 sources or more in the order of its last
                                forward iteration counts, fewest first, so that a barrier group

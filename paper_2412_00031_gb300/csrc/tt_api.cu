@@ -101,12 +101,6 @@ constexpr int kFlagInts = 6;
 constexpr size_t kCoefBudgetBytes = 64ull << 30;
 // Largest factor cache (1/T0 and grad T0 / T0 per node and source) one forward slice keeps.
 constexpr size_t kFactorCacheBudgetBytes = 32ull << 30;
-// Barrier groups that one face-adjoint launch runs side by side.
-#ifndef TTGB_ADJ_GROUPS
-#define TTGB_ADJ_GROUPS 4
-#endif
-constexpr int kAdjGroups = TTGB_ADJ_GROUPS;
-
 tt_status fail(tt_ctx *c, tt_status s, const char *fmt, ...) {
     if (c) {
         va_list ap;
@@ -859,42 +853,9 @@ tt_status enq_adjoint(tt_ctx *ctx, Work<F> &W, const tt_model *m, int B, const v
     // Face-coefficient sweep when the per-(node, source) coefficients fit the workspace
     // budget; otherwise the sweep that evaluates the flux velocities at every update.
     const bool faces = W.coef_ok;
-    int grid, block, slots;
-    int n_bgroups = 1, grp_blocks = 0, grp_src = B, adj_launch_groups = 1;
-    if (faces) {
-        // Source slices of adj_chunk sources, one cooperative launch each, run one after
-        // another: a hyperplane of one slice (coefficients of two planes, P of three) then
-        // stays in L2. Automatic: slices of at most 128 sources.
-        // Each launch covers `chunk` sources (default: all), split into up to
-        // TTGB_ADJ_GROUPS barrier groups of >= 64 sources that run side by side.
-        block = 256;
-        int chunk = o->adj_chunk > 0 ? o->adj_chunk : B;
-        chunk = chunk >= B ? B : (chunk + 31) / 32 * 32;
-        int groups = o->adj_groups > 0 ? o->adj_groups : (chunk + 63) / 64;
-        if (o->adj_groups <= 0 && groups > kAdjGroups) groups = kAdjGroups;
-        if (groups > (chunk + 31) / 32) groups = (chunk + 31) / 32;  // >= 32 sources a group
-        grp_src = ((chunk + groups - 1) / groups + 31) / 32 * 32;
-        groups = (chunk + grp_src - 1) / grp_src;
-        n_bgroups = (B + grp_src - 1) / grp_src;  // groups over the whole batch
-        adj_launch_groups = groups;
-        size_t smem = (size_t)grp_src * 2 * sizeof(F);
-        int per_sm = adjoint_faces_blocks_per_sm<F>(block, smem);
-        if (per_sm <= 0) return fail(ctx, TT_ECUDA, "adjoint sweep cannot be resident");
-        if (per_sm > 4) per_sm = 4;
-        int max_grid = per_sm * ctx->n_sm;
-        if (o->launch_blocks > 0 && o->launch_blocks < max_grid) max_grid = o->launch_blocks;
-        grp_blocks = max_grid / groups;
-        if ((long long)grp_blocks * block < grp_src) {
-            int need = (grp_src + block - 1) / block;
-            if ((long long)need * groups > (long long)per_sm * ctx->n_sm)
-                return fail(ctx, TT_EINVAL, "batch of %d sources exceeds one resident launch", B);
-            grp_blocks = need;
-        }
-        grid = grp_blocks * groups;
-        slots = 0;
-    } else if ((s = sweep_shape<F>(ctx, B, ctx->full, o->launch_blocks, grid, block, slots)) != TT_OK) {
+    int grid = 0, block = 0, slots = 0;
+    if (!faces && (s = sweep_shape<F>(ctx, B, ctx->full, o->launch_blocks, grid, block, slots)) != TT_OK)
         return s;
-    }
     const GeoTab<F> &t = geo<F>(ctx);
     AdjArgs<F> a;
     memset(&a, 0, sizeof a);
@@ -925,19 +886,27 @@ tt_status enq_adjoint(tt_ctx *ctx, Work<F> &W, const tt_model *m, int B, const v
     a.max_iter = o->max_iter_adj;
     a.spin_ns = spin_ns(o);
     a.coef = faces ? reinterpret_cast<F *>(W.coef) : nullptr;
-    a.n_bgroups = n_bgroups;
-    a.grp_blocks = grp_blocks;
-    a.grp_src = grp_src;
+    a.src_lo = 0;
+    a.src_n = B;
     if (faces) {
         CK(launch_adjoint_coefs<F>(a, ctx->st));
         ctx->launches += 1;
     }
     CK(record(ctx, ctx->ev_start[TT_STATS_ADJOINT]));
     if (faces) {
-        for (int q = 0; q < n_bgroups; q += adj_launch_groups) {
-            a.grp_base = q;
-            const int ng = n_bgroups - q < adj_launch_groups ? n_bgroups - q : adj_launch_groups;
-            CK(launch_adjoint_faces<F>(a, grp_blocks * ng, block, ctx->st));
+        // slices of adj_chunk sources (automatic: all), one launch each, one after another
+        const int chunk = o->adj_chunk > 0 && o->adj_chunk < B ? (o->adj_chunk + 31) / 32 * 32 : B;
+        for (int q = 0; q < B; q += chunk) {
+            a.src_lo = q;
+            a.src_n = chunk < B - q ? chunk : B - q;
+            int gr = 0, bl = 0;
+            const cudaError_t e = run_plane_adjoint<F>(a, o->adj_groups, W.partial, ctx->n_sm,
+                                                       o->launch_blocks, &gr, &bl, ctx->st);
+            if (e == cudaErrorInvalidConfiguration)
+                return fail(ctx, TT_EINVAL, "batch of %d sources exceeds one resident launch", B);
+            CK(e);
+            grid = gr > grid ? gr : grid;
+            block = bl > block ? bl : block;
             ctx->launches += 1;
         }
     } else {

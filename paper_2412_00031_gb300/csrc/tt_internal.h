@@ -93,8 +93,7 @@ template <typename F> struct AdjArgs {
     // Face coefficients, four planes of [N][B] (plane stride N * B): A a / delta on the +r,
     // +theta, +phi faces and J_c S_c (NaN on the source's fixed set)
     F *coef;
-    int n_bgroups, grp_blocks, grp_src;  // barrier groups (as in FwdArgs)
-    int grp_base;              // group index of this launch's first group
+    int src_lo, src_n;         // sources of this launch
     const unsigned int *nodes;
     const int *off;
     BarrierState *bar;
@@ -155,8 +154,10 @@ constexpr int kMaxBarrierGroups = 8;
 template <typename F> int adjoint_blocks_per_sm(int block, size_t smem);
 // Face-coefficient adjoint: coefficients once per solve, then the sweep over P.
 template <typename F> cudaError_t launch_adjoint_coefs(const AdjArgs<F> &a, cudaStream_t st);
-template <typename F> cudaError_t launch_adjoint_faces(const AdjArgs<F> &a, int grid, int block,
-                                                       cudaStream_t st);
-template <typename F> int adjoint_faces_blocks_per_sm(int block, size_t smem);
+// The sweep from the coefficients (tt_plane.cu) for the sources [src_lo, src_lo + src_n) of a; emax:
+// 6 * src_n values of F. cudaErrorInvalidConfiguration: they exceed one resident launch.
+template <typename F>
+cudaError_t run_plane_adjoint(AdjArgs<F> a, int groups, F *emax, int n_sm, int launch_blocks, int *grid,
+                              int *block, cudaStream_t st);
 
 }  // namespace ttgb

@@ -29,29 +29,12 @@
 // prefetch of them, a warp of its own for the barrier, four sources a thread: all slower.
 #include <cuda_runtime.h>
 
-#include <algorithm>
-#include <cstring>
-
-#include "tt_internal.h"
+#include "tt_plane.cuh"
 #include "tt_update.cuh"
 
 namespace ttgb {
 
 namespace {
-
-// NS neighbouring sources of one node: one load or store.
-__device__ __forceinline__ void ld_pack(const float *p, float (&v)[1]) { v[0] = *p; }
-__device__ __forceinline__ void ld_pack(const double *p, double (&v)[1]) { v[0] = *p; }
-__device__ __forceinline__ void ld_pack(const float *p, float (&v)[2]) {
-    const float2 t = *reinterpret_cast<const float2 *>(p);
-    v[0] = t.x;
-    v[1] = t.y;
-}
-__device__ __forceinline__ void st_pack(float *p, const float (&v)[1]) { *p = v[0]; }
-__device__ __forceinline__ void st_pack(double *p, const double (&v)[1]) { *p = v[0]; }
-__device__ __forceinline__ void st_pack(float *p, const float (&v)[2]) {
-    *reinterpret_cast<float2 *>(p) = make_float2(v[0], v[1]);
-}
 
 __device__ __forceinline__ NodeRec<float> ld_rec(const NodeRec<float> *r) {
     const float4 a = __ldg(reinterpret_cast<const float4 *>(r)), b = __ldg(reinterpret_cast<const float4 *>(r) + 1);
@@ -116,21 +99,11 @@ template <typename F, int SCHEME, int NS> struct Update {
     }
 };
 
-// A node of an ordering, and the planes of a time step: of orderings o0, o0 + 1, o0 + 2 the first
-// list entry q and the count c.
+// A node of an ordering.
 struct Node {
     int i, j, k, aa, bb, cc;
     long long n;
 };
-struct Planes {
-    int o0, q[3], c[3];
-    __device__ __forceinline__ int total() const { return c[0] + c[1] + c[2]; }
-};
-
-// Threads of an SM: 80 registers a thread. Fewer threads of more registers are slower, also where
-// they would not spill (the Godunov updates): 121x161x161 x 256 sources 639 / 543 / 494 / 482 ms
-// with 384 / 512 / 640 / 768.
-constexpr int kPlaneThreads = 768;
 
 template <typename F, int SCHEME, int NS>
 __global__ void __launch_bounds__(kPlaneThreads, 1)
@@ -165,21 +138,13 @@ __global__ void __launch_bounds__(kPlaneThreads, 1)
     const unsigned nblk = (unsigned)m.grp_blocks;
     const long long osp = B, ost = (long long)g.np * B, osr = (long long)g.nt * g.np * B;
     using U = Update<F, SCHEME, NS>;
+    const PlaneSched sch{s_off, s_start, a.nodes, a.n_planes, m.steps};
 
     for (int it = 0; it < a.max_iter; ++it) {
         // The sources that still iterate (NS to a thread), so that no thread is kept for converged
         // ones: a solve's last iterations have few sources, in any order of the batch.
         if (threadIdx.x < 32) {
-            int n = 0;
-            for (int u0 = 0; u0 < Bg / NS; u0 += 32) {
-                const int u = u0 + (int)threadIdx.x;
-                bool on = false;
-#pragma unroll
-                for (int h = 0; h < NS; ++h) on = on || (u < Bg / NS && s_on[u * NS + h]);
-                const unsigned mask = __ballot_sync(0xffffffffu, on);
-                if (on) s_list[n + __popc(mask & ((1u << threadIdx.x) - 1u))] = u;
-                n += __popc(mask);
-            }
+            const int n = plane_units<NS>(s_on, Bg / NS, s_list);
             if (threadIdx.x == 0) s_units = n;
         }
         __syncthreads();
@@ -202,26 +167,6 @@ __global__ void __launch_bounds__(kPlaneThreads, 1)
         // static: the next entry is looked up while a node is updated, the next time step's first
         // one before the barrier.
         Planes cp, np;
-        auto planes = [&](Planes &d, int tau, int o0) {
-            if (tau - s_start[o0] >= a.n_planes && o0 < 7) ++o0;
-            d.o0 = o0;
-#pragma unroll
-            for (int u = 0; u < 3; ++u) {
-                const int o = o0 + u, L = tau - s_start[o & 7];
-                d.q[u] = 0;
-                d.c[u] = 0;
-                if (o < 8 && tau < m.steps && L >= 0 && L < a.n_planes) {
-                    d.q[u] = s_off[L];
-                    d.c[u] = s_off[L + 1] - d.q[u];
-                }
-            }
-        };
-        auto entry = [&](const Planes &d, int x, int &o) {
-            const int u = x < d.c[0] ? 0 : x < d.c[0] + d.c[1] ? 1 : 2;
-            o = d.o0 + u;
-            const int q = u == 0 ? d.q[0] + x : u == 1 ? d.q[1] + (x - d.c[0]) : d.q[2] + (x - d.c[0] - d.c[1]);
-            return __ldg(a.nodes + q);
-        };
         auto place = [&](int o, unsigned pk) {
             Node d;
             d.aa = (int)(pk >> 20) & 1023;
@@ -233,11 +178,11 @@ __global__ void __launch_bounds__(kPlaneThreads, 1)
             d.n = ((long long)d.i * g.nt + d.j) * g.np + d.k;
             return d;
         };
-        planes(cp, 0, 0);
+        sch.planes(cp, 0, 0);
         int o = 0;
         unsigned pk = 0;
         if (any && slot < cp.total()) {
-            pk = entry(cp, slot, o);
+            pk = sch.entry(cp, slot, o);
         }
         // the stencil, factors and record of the node in hand, and where it is
         F v[7][NS];
@@ -264,16 +209,16 @@ __global__ void __launch_bounds__(kPlaneThreads, 1)
             if (mine) load();
             // the next time step's planes and this thread's first node there: static, and looked
             // up while the loads above are on their way
-            planes(np, tau + 1, cp.o0);
+            sch.planes(np, tau + 1, cp.o0);
             int on = 0;
             unsigned pkn = 0;
-            if (any && slot < np.total()) pkn = entry(np, slot, on);
+            if (any && slot < np.total()) pkn = sch.entry(np, slot, on);
             if (mine)
                 for (int x = slot;;) {
                     const bool rr = o & 4, rt = o & 2, rp = o & 1;
                     const bool face = pk & 0x40000000u;
                     x += slots;
-                    if (x < total) pk = entry(cp, x, o);
+                    if (x < total) pk = sch.entry(cp, x, o);
                     F tn[NS];
                     U::run(fc, v, rec, a.er, act, tn, err);
                     // values that keep their bits are not stored: their line stays clean
@@ -407,22 +352,165 @@ template <typename F> __global__ void edge_kernel(FwdArgs<F> a, int axis) {
     *p = fmax_((F)2 * t1 - t2, t2);
 }
 
-}  // namespace
+// The adjoint sweep (Eq. 5) from the face coefficients (adj_coef_kernel, face_update), over every
+// node, in the same organisation; no faces to complete. emax: [3][2][src_n], by iteration mod 3 the
+// sources' largest |change| of P and, in the last ordering, largest |P|.
+template <typename F, int NS>
+__global__ void __launch_bounds__(kPlaneThreads, 1) adj_plane_kernel(AdjArgs<F> a, PlaneShape m, F *emax) {
+    extern __shared__ __align__(8) int s_off[];
+    __shared__ int s_units, s_start[8];
+    const GridC &g = a.g;
+    const long long B = a.B;
+    const int grp = blockIdx.x / m.grp_blocks, blk = blockIdx.x - grp * m.grp_blocks;
+    const int src0 = grp * m.grp_src;                              // within the launch's sources
+    const int Bg = min(a.src_n, src0 + m.grp_src) - src0;
+    if (Bg <= 0) return;
+    barrier_begin();
+    F *s_err = reinterpret_cast<F *>(s_off + (a.n_planes + 2) / 2 * 2), *s_pm = s_err + Bg;
+    int *s_list = reinterpret_cast<int *>(s_pm + Bg);
+    unsigned char *s_on = reinterpret_cast<unsigned char *>(s_list + Bg);
+    for (int q = threadIdx.x; q <= a.n_planes; q += blockDim.x) s_off[q] = a.off[q];
+    for (int q = threadIdx.x; q < Bg; q += blockDim.x) s_on[q] = 1;
+    if (threadIdx.x == 0)
+#pragma unroll
+        for (int o = 0; o < 8; ++o) s_start[o] = m.start[o];
+    __syncthreads();
+    const long long tid = ((long long)(threadIdx.x >> 5) * m.grp_blocks + blk) * 32 + (threadIdx.x & 31);
+    BarrierState *bar = a.bar + grp;
+    const unsigned nblk = (unsigned)m.grp_blocks;
+    const long long sp = B, st = (long long)g.np * B, sr = (long long)g.nt * g.np * B;
+    const long long plane = g.N * B;                               // coefficient plane stride
+    const PlaneSched sch{s_off, s_start, a.nodes, a.n_planes, m.steps};
 
-// Start times of the 8 orderings of an iteration: o + 1 flips the axes of the bits that change.
-// At most three orderings are in progress at a time.
-static void plane_starts(PlaneShape &m, int na, int nb, int nc) {
-    const int planes = na + nb + nc - 2;
-    m.start[0] = 0;
-    for (int o = 1; o < 8; ++o) {
-        const int f = o ^ (o - 1);
-        int d = 2 + (f & 4 ? na - 1 : 0) + (f & 2 ? nb - 1 : 0) + (f & 1 ? nc - 1 : 0);
-        if (d > planes) d = planes;
-        m.start[o] = m.start[o - 1] + d;
-        if (o >= 3 && m.start[o] < m.start[o - 3] + planes) m.start[o] = m.start[o - 3] + planes;
+    for (int it = 0; it < a.max_iter; ++it) {
+        if (threadIdx.x < 32) {
+            const int n = plane_units<NS>(s_on, Bg / NS, s_list);
+            if (threadIdx.x == 0) s_units = n;
+        }
+        for (int q = threadIdx.x; q < Bg; q += blockDim.x) s_err[q] = s_pm[q] = 0;
+        __syncthreads();
+        const int lanes = s_units;
+        if (lanes == 0) break;
+        const int slots = (int)(((long long)m.grp_blocks * blockDim.x) / lanes);
+        const bool any = tid < (long long)slots * lanes;
+        const int slot = any ? (int)(tid / lanes) : 0;
+        const int bl = src0 + (any ? s_list[tid - (long long)slot * lanes] * NS : 0);
+        const int b = a.src_lo + bl;
+        const F *cX = a.coef, *cY = a.coef + plane, *cZ = a.coef + 2 * plane, *cW = a.coef + 3 * plane;
+        bool act[NS];
+        F err[NS], pmax[NS];
+#pragma unroll
+        for (int h = 0; h < NS; ++h) {
+            act[h] = any && s_on[bl - src0 + h];
+            err[h] = pmax[h] = 0;
+        }
+        Planes cp, np;
+        sch.planes(cp, 0, 0);
+        int o = 0;
+        unsigned pk = 0;
+        if (any && slot < cp.total()) pk = sch.entry(cp, slot, o);
+        F w[NS], cx[NS], cy[NS], cz[NS], mx[NS], my[NS], mz[NS], Pn[6][NS], po[NS];
+        long long x = 0;
+        bool last = false;
+        auto load = [&]() {
+            const int aa = (int)(pk >> 20) & 1023, bb = (int)(pk >> 10) & 1023, cc = (int)pk & 1023;
+            const int i = o & 4 ? g.nr - 1 - aa : aa, j = o & 2 ? g.nt - 1 - bb : bb, k = o & 1 ? g.np - 1 - cc : cc;
+            x = node_index(g, i, j, k) * B + b;
+            last = o == 7;
+            ld_pack(cW + x, w);
+            ld_pack(cX + x, cx);
+            ld_pack(cY + x, cy);
+            ld_pack(cZ + x, cz);
+            ld_pack(a.P + x, po);
+            // no flux through the outer faces: zero coefficients and values there
+            const bool hr = i < g.nr - 1, lr = i > 0, ht = j < g.nt - 1, lt = j > 0, hp = k < g.np - 1, lp = k > 0;
+#pragma unroll
+            for (int h = 0; h < NS; ++h) {
+                mx[h] = my[h] = mz[h] = 0;
+#pragma unroll
+                for (int q = 0; q < 6; ++q) Pn[q][h] = 0;
+            }
+            if (lr) ld_pack(cX + x - sr, mx);
+            if (lt) ld_pack(cY + x - st, my);
+            if (lp) ld_pack(cZ + x - sp, mz);
+            if (hr) ld_pack(a.P + x + sr, Pn[0]);
+            if (lr) ld_pack(a.P + x - sr, Pn[1]);
+            if (ht) ld_pack(a.P + x + st, Pn[2]);
+            if (lt) ld_pack(a.P + x - st, Pn[3]);
+            if (hp) ld_pack(a.P + x + sp, Pn[4]);
+            if (lp) ld_pack(a.P + x - sp, Pn[5]);
+        };
+        for (int tau = 0; tau < m.steps; ++tau) {
+            const int total = cp.total();
+            const bool mine = any && slot < total;
+            if (mine) load();
+            sch.planes(np, tau + 1, cp.o0);
+            int on = 0;
+            unsigned pkn = 0;
+            if (any && slot < np.total()) pkn = sch.entry(np, slot, on);
+            if (mine)
+                for (int q = slot;;) {
+                    q += slots;
+                    if (q < total) pk = sch.entry(cp, q, o);
+                    F pn[NS];
+                    bool moved = false;
+#pragma unroll
+                    for (int h = 0; h < NS; ++h) {
+                        pn[h] = po[h];
+                        // the fixed set (w is NaN) and a converged source keep their values
+                        if (act[h] && w[h] == w[h]) {
+                            const F nb[6] = {Pn[0][h], Pn[1][h], Pn[2][h], Pn[3][h], Pn[4][h], Pn[5][h]};
+                            pn[h] = face_update<F>(cx[h], cy[h], cz[h], w[h], mx[h], my[h], mz[h], nb);
+                            err[h] = fmax_(err[h], fabs(pn[h] - po[h]));
+                            if (last) pmax[h] = fmax_(pmax[h], fabs(pn[h]));
+                        }
+                        moved = moved || bits_of(pn[h]) != bits_of(po[h]);
+                    }
+                    if (moved) st_pack(a.P + x, pn);
+                    if (q >= total) break;
+                    load();
+                }
+            if (!grid_barrier(bar, a.spin_ns, nblk)) return;
+            o = on;
+            pk = pkn;
+            cp = np;
+        }
+        // the sources' maxima: over the block, then over the group's blocks
+        F *e = emax + (long long)(it % 3) * 2 * a.src_n;
+#pragma unroll
+        for (int h = 0; h < NS; ++h)
+            if (act[h]) {
+                atomic_max_nonneg(&s_err[bl - src0 + h], err[h]);
+                atomic_max_nonneg(&s_pm[bl - src0 + h], pmax[h]);
+            }
+        __syncthreads();
+        for (int q = threadIdx.x; q < Bg; q += blockDim.x)
+            if (s_on[q]) {
+                atomic_max_nonneg(e + src0 + q, s_err[q]);
+                atomic_max_nonneg(e + a.src_n + src0 + q, s_pm[q]);
+            }
+        if (!grid_barrier(bar, a.spin_ns, nblk)) return;
+        // every block evaluates the stopping rule; the group's first one reports, and clears the
+        // maxima of the iteration after the next
+        F *e2 = emax + (long long)((it + 2) % 3) * 2 * a.src_n;
+        for (int q = threadIdx.x; q < Bg; q += blockDim.x) {
+            const int s = src0 + q;
+            const bool done = ((volatile F *)e)[s] <= a.tol * ((volatile F *)e)[a.src_n + s];
+            if (blk == 0) {
+                if (s_on[q]) {
+                    a.iters[a.src_lo + s] = it + 1;
+                    if (done) a.conv[a.src_lo + s] = 1;
+                }
+                e2[s] = e2[a.src_n + s] = 0;
+            }
+            if (done) s_on[q] = 0;
+        }
+        __syncthreads();
     }
-    m.steps = m.start[7] + planes;
+    barrier_end(bar, nblk);
 }
+
+}  // namespace
 
 template <typename F>
 cudaError_t run_plane_forward(FwdArgs<F> a, int groups, int *moved, int n_sm, int launch_blocks, int *grid,
@@ -430,53 +518,18 @@ cudaError_t run_plane_forward(FwdArgs<F> a, int groups, int *moved, int n_sm, in
     cudaError_t e;
     const int n = a.src_n;
     const bool tele = a.scheme == 3;
-    int threads = kPlaneThreads;
     PlaneShape m;
     memset(&m, 0, sizeof m);
     plane_starts(m, a.na, a.nb, a.nc);
-    // Pairs of sources (FP32, every row whole aligned pairs) where a time step has more updates
-    // than the GPU holds threads: half the instructions and loads an update. Below that a thread
-    // per source has the shorter time step. LF, ms per 2 iterations, single / pairs: 81^3 x 16
-    // sources 6.81 / 6.97, x 32 8.32 / 7.86, x 100 14.2 / 12.1; 121x161x161 x 32 26.6 / 23.0.
-    const double per_step = 8.0 * a.na * a.nb * a.nc / m.steps * n;
+    // pairs need FP32 and rows of whole aligned pairs
     const bool pair = sizeof(F) == 4 && n % 2 == 0 && a.B % 2 == 0 && a.src_lo % 2 == 0 &&
-                      (size_t)a.tau % 8 == 0 && per_step > (double)threads * n_sm;
-    const int ns = pair ? 2 : 1;
+                      (size_t)a.tau % 8 == 0 && plane_pairs(m, a.na, a.nb, a.nc, n, n_sm);
     const void *fn = plane_ptr<F, 1>(a.scheme);
     if constexpr (sizeof(F) == 4)
         if (pair) fn = plane_ptr<F, 2>(a.scheme);
     const size_t smem = sizeof(int) * (a.n_planes + 1 + 2 * (size_t)n) + n;
-    if ((e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess)
+    if ((e = plane_shape(m, fn, smem, a.na, a.nb, a.nc, n, pair ? 2 : 1, groups, n_sm, launch_blocks, grid, block)) != cudaSuccess)
         return e;
-    // one block an SM and group, so that a barrier has as few arrivals as there are SMs (a barrier
-    // of 608 blocks takes 2.5 us, of 152 1.6 us); groups only where asked for
-    if (groups <= 0) groups = 1;
-    if (groups > kMaxBarrierGroups) groups = kMaxBarrierGroups;
-    if (groups > (n + 31) / 32) groups = (n + 31) / 32;
-    threads = threads / groups / 32 * 32;
-    // no more threads than the widest plane has nodes and sources
-    const int ext[3] = {a.na, a.nb, a.nc};
-    long long widest = 0;
-    for (int x = 0; x < 3; ++x)
-        for (int y = x + 1; y < 3; ++y) widest = std::max(widest, (long long)ext[x] * ext[y]);
-    const long long want = (widest * (n / ns) / groups / n_sm + 31) / 32 * 32;
-    if (want < threads) threads = want < 32 ? 32 : (int)want;
-    int per_sm = 0;
-    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, threads, smem)) != cudaSuccess) return e;
-    if (per_sm <= 0) return cudaErrorInvalidConfiguration;
-    if (per_sm > groups) per_sm = groups;
-    int most = per_sm * n_sm;
-    if (launch_blocks > 0 && launch_blocks < most) most = launch_blocks;
-    if (groups > most) groups = most;
-    m.grp_src = ((n + groups - 1) / groups + ns - 1) / ns * ns;
-    groups = (n + m.grp_src - 1) / m.grp_src;
-    m.grp_blocks = most / groups;
-    // a group's blocks hold at least one thread per source
-    const int need = (m.grp_src / ns + threads - 1) / threads;
-    if (m.grp_blocks < need) m.grp_blocks = need;
-    if ((long long)m.grp_blocks * groups > (long long)per_sm * n_sm) return cudaErrorInvalidConfiguration;
-    *grid = m.grp_blocks * groups;
-    *block = threads;
     *kernels = tele ? 1 : 4;
     m.moved = moved;
     if ((e = cudaMemsetAsync(moved, 0, sizeof(int) * 3 * (size_t)n, st)) != cudaSuccess) return e;
@@ -489,7 +542,7 @@ cudaError_t run_plane_forward(FwdArgs<F> a, int groups, int *moved, int n_sm, in
         if (!pair && (e = launch_t0_cache<F>(a, st)) != cudaSuccess) return e;
     }
     void *args[] = {&a, &m};
-    if ((e = cudaLaunchCooperativeKernel(fn, dim3(*grid), dim3(threads), args, smem, st)) != cudaSuccess) return e;
+    if ((e = cudaLaunchCooperativeKernel(fn, dim3(*grid), dim3(*block), args, smem, st)) != cudaSuccess) return e;
     if (!tele)
         for (int axis = 1; axis <= 2; ++axis) {
             const long long q = (axis == 1 ? 4LL * a.g.np : 4LL * (a.g.nr + a.g.nt - 2)) * n;
@@ -498,6 +551,29 @@ cudaError_t run_plane_forward(FwdArgs<F> a, int groups, int *moved, int n_sm, in
     return cudaGetLastError();
 }
 
+template <typename F>
+cudaError_t run_plane_adjoint(AdjArgs<F> a, int groups, F *emax, int n_sm, int launch_blocks, int *grid,
+                              int *block, cudaStream_t st) {
+    cudaError_t e;
+    const int n = a.src_n;
+    PlaneShape m;
+    memset(&m, 0, sizeof m);
+    plane_starts(m, a.g.nr, a.g.nt, a.g.np);
+    const bool pair = sizeof(F) == 4 && n % 2 == 0 && a.B % 2 == 0 && a.src_lo % 2 == 0 &&
+                      (size_t)a.P % 8 == 0 && plane_pairs(m, a.g.nr, a.g.nt, a.g.np, n, n_sm);
+    const void *fn = (const void *)adj_plane_kernel<F, 1>;
+    if constexpr (sizeof(F) == 4)
+        if (pair) fn = (const void *)adj_plane_kernel<F, 2>;
+    const size_t smem = sizeof(int) * (a.n_planes + 2 + (size_t)n) + 2 * sizeof(F) * (size_t)n + n;
+    if ((e = plane_shape(m, fn, smem, a.g.nr, a.g.nt, a.g.np, n, pair ? 2 : 1, groups, n_sm, launch_blocks, grid, block)) != cudaSuccess)
+        return e;
+    if ((e = cudaMemsetAsync(emax, 0, sizeof(F) * 6 * (size_t)n, st)) != cudaSuccess) return e;
+    void *args[] = {&a, &m, &emax};
+    return cudaLaunchCooperativeKernel(fn, dim3(*grid), dim3(*block), args, smem, st);
+}
+
+template cudaError_t run_plane_adjoint<float>(AdjArgs<float>, int, float *, int, int, int *, int *, cudaStream_t);
+template cudaError_t run_plane_adjoint<double>(AdjArgs<double>, int, double *, int, int, int *, int *, cudaStream_t);
 template cudaError_t run_plane_forward<float>(FwdArgs<float>, int, int *, int, int, int *, int *, int *, cudaStream_t);
 template cudaError_t run_plane_forward<double>(FwdArgs<double>, int, int *, int, int, int *, int *, int *, cudaStream_t);
 

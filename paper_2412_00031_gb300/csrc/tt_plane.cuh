@@ -1,0 +1,143 @@
+// What the plane sweeps (tt_plane.cu: forward, adjoint) share: the planes of a time step, the list of
+// sources that still iterate, the vector accesses of a thread's sources and the launch shape.
+#pragma once
+
+#include <algorithm>
+#include <cstring>
+
+#include "tt_internal.h"
+
+namespace ttgb {
+
+// Threads of an SM: 80 registers a thread. Fewer threads of more registers are slower, also where
+// they would not spill (the Godunov updates): 121x161x161 x 256 sources 639 / 543 / 494 / 482 ms
+// with 384 / 512 / 640 / 768.
+constexpr int kPlaneThreads = 768;
+
+// NS neighbouring sources of one node: one load or store.
+__device__ __forceinline__ void ld_pack(const float *p, float (&v)[1]) { v[0] = *p; }
+__device__ __forceinline__ void ld_pack(const double *p, double (&v)[1]) { v[0] = *p; }
+__device__ __forceinline__ void ld_pack(const float *p, float (&v)[2]) {
+    const float2 t = *reinterpret_cast<const float2 *>(p);
+    v[0] = t.x;
+    v[1] = t.y;
+}
+__device__ __forceinline__ void st_pack(float *p, const float (&v)[1]) { *p = v[0]; }
+__device__ __forceinline__ void st_pack(double *p, const double (&v)[1]) { *p = v[0]; }
+__device__ __forceinline__ void st_pack(float *p, const float (&v)[2]) {
+    *reinterpret_cast<float2 *>(p) = make_float2(v[0], v[1]);
+}
+
+// The planes of a time step: of orderings o0, o0 + 1, o0 + 2 the first list entry q and the count c.
+struct Planes {
+    int o0, q[3], c[3];
+    __device__ __forceinline__ int total() const { return c[0] + c[1] + c[2]; }
+};
+
+// The schedule of an iteration: off (shared memory) and nodes as in Schedule, start (shared
+// memory) the orderings' first time steps.
+struct PlaneSched {
+    const int *off, *start;
+    const unsigned *nodes;
+    int n_planes, steps;
+    // the planes of time step tau; o0: the first ordering in progress one step before
+    __device__ __forceinline__ void planes(Planes &d, int tau, int o0) const {
+        if (tau - start[o0] >= n_planes && o0 < 7) ++o0;
+        d.o0 = o0;
+#pragma unroll
+        for (int u = 0; u < 3; ++u) {
+            const int o = o0 + u, L = tau - start[o & 7];
+            d.q[u] = 0;
+            d.c[u] = 0;
+            if (o < 8 && tau < steps && L >= 0 && L < n_planes) {
+                d.q[u] = off[L];
+                d.c[u] = off[L + 1] - d.q[u];
+            }
+        }
+    }
+    // node x of the concatenated planes and its ordering
+    __device__ __forceinline__ unsigned entry(const Planes &d, int x, int &o) const {
+        const int u = x < d.c[0] ? 0 : x < d.c[0] + d.c[1] ? 1 : 2;
+        o = d.o0 + u;
+        return __ldg(nodes + (u == 0 ? d.q[0] + x : u == 1 ? d.q[1] + (x - d.c[0]) : d.q[2] + (x - d.c[0] - d.c[1])));
+    }
+};
+
+// list = the units of NS sources of which one is on, in order; returns their number. One warp.
+template <int NS> __device__ __forceinline__ int plane_units(const unsigned char *on_, int units, int *list) {
+    int n = 0;
+    const int lane = threadIdx.x & 31;
+    for (int u0 = 0; u0 < units; u0 += 32) {
+        const int u = u0 + lane;
+        bool on = false;
+#pragma unroll
+        for (int h = 0; h < NS; ++h) on = on || (u < units && on_[u * NS + h]);
+        const unsigned mask = __ballot_sync(0xffffffffu, on);
+        if (on) list[n + __popc(mask & ((1u << lane) - 1u))] = u;
+        n += __popc(mask);
+    }
+    return n;
+}
+
+// Start times of the 8 orderings of an iteration over a box na x nb x nc: o + 1 flips the axes of
+// the bits that change. At most three orderings are in progress at a time.
+inline void plane_starts(PlaneShape &m, int na, int nb, int nc) {
+    const int planes = na + nb + nc - 2;
+    m.start[0] = 0;
+    for (int o = 1; o < 8; ++o) {
+        const int f = o ^ (o - 1);
+        int d = 2 + (f & 4 ? na - 1 : 0) + (f & 2 ? nb - 1 : 0) + (f & 1 ? nc - 1 : 0);
+        if (d > planes) d = planes;
+        m.start[o] = m.start[o - 1] + d;
+        if (o >= 3 && m.start[o] < m.start[o - 3] + planes) m.start[o] = m.start[o - 3] + planes;
+    }
+    m.steps = m.start[7] + planes;
+}
+
+// Pairs of sources where a time step has more updates than the GPU holds threads: half the
+// instructions and loads an update. Below that a thread per source has the shorter time step.
+// Forward LF, ms per 2 iterations, single / pairs: 81^3 x 16 sources 6.81 / 6.97, x 32 8.32 /
+// 7.86, x 100 14.2 / 12.1; 121x161x161 x 32 26.6 / 23.0.
+inline bool plane_pairs(const PlaneShape &m, int na, int nb, int nc, int n, int n_sm) {
+    return 8.0 * na * nb * nc / m.steps * n > (double)kPlaneThreads * n_sm;
+}
+
+// Blocks, threads and barrier groups (0 = 1) for n sources, ns to a thread; smem: dynamic shared
+// memory. One block an SM and group, so that a barrier has as few arrivals as there are SMs (a
+// barrier of 608 blocks takes 2.5 us, of 152 1.6 us); no more threads than the widest plane has
+// nodes and sources. cudaErrorInvalidConfiguration: the sources exceed one resident launch.
+inline cudaError_t plane_shape(PlaneShape &m, const void *fn, size_t smem, int na, int nb, int nc, int n, int ns,
+                               int groups, int n_sm, int launch_blocks, int *grid, int *block) {
+    cudaError_t e;
+    if ((e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess)
+        return e;
+    if (groups <= 0) groups = 1;
+    if (groups > kMaxBarrierGroups) groups = kMaxBarrierGroups;
+    if (groups > (n + 31) / 32) groups = (n + 31) / 32;
+    int threads = kPlaneThreads / groups / 32 * 32;
+    const int ext[3] = {na, nb, nc};
+    long long widest = 0;
+    for (int x = 0; x < 3; ++x)
+        for (int y = x + 1; y < 3; ++y) widest = std::max(widest, (long long)ext[x] * ext[y]);
+    const long long want = (widest * (n / ns) / groups / n_sm + 31) / 32 * 32;
+    if (want < threads) threads = want < 32 ? 32 : (int)want;
+    int per_sm = 0;
+    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, threads, smem)) != cudaSuccess) return e;
+    if (per_sm <= 0) return cudaErrorInvalidConfiguration;
+    if (per_sm > groups) per_sm = groups;
+    int most = per_sm * n_sm;
+    if (launch_blocks > 0 && launch_blocks < most) most = launch_blocks;
+    if (groups > most) groups = most;
+    m.grp_src = ((n + groups - 1) / groups + ns - 1) / ns * ns;
+    groups = (n + m.grp_src - 1) / m.grp_src;
+    m.grp_blocks = most / groups;
+    // a group's blocks hold at least one thread per source
+    const int need = (m.grp_src / ns + threads - 1) / threads;
+    if (m.grp_blocks < need) m.grp_blocks = need;
+    if ((long long)m.grp_blocks * groups > (long long)per_sm * n_sm) return cudaErrorInvalidConfiguration;
+    *grid = m.grp_blocks * groups;
+    *block = threads;
+    return cudaSuccess;
+}
+
+}  // namespace ttgb

@@ -15,14 +15,6 @@
 
 namespace ttgb {
 
-__device__ __forceinline__ void atomic_max_nonneg(float *p, float v) {
-    atomicMax(reinterpret_cast<unsigned int *>(p), __float_as_uint(v));
-}
-__device__ __forceinline__ void atomic_max_nonneg(double *p, double v) {
-    atomicMax(reinterpret_cast<unsigned long long *>(p),
-              (unsigned long long)__double_as_longlong(v));
-}
-
 __device__ __forceinline__ unsigned smem_u32(const void *p) {
     return (unsigned)__cvta_generic_to_shared(p);
 }
@@ -974,176 +966,6 @@ template <typename F> __global__ void adj_coef_kernel(AdjArgs<F> a) {
     }
 }
 
-// Upwind update of one (node, source) from its face coefficients (Eq. 5 discretised as in
-// adj_update): c = (+r, +theta, +phi face coefficients, J S), cm = the -r, -theta, -phi
-// neighbours' plus-face coefficients, Pn = P at (+r, -r, +theta, -theta, +phi, -phi).
-// Rounding-explicit, so both lanes' copies give identical bits.
-template <typename F>
-__device__ __forceinline__ F face_update(F cx, F cy, F cz, F cw, F cmx, F cmy, F cmz,
-                                         const F (&Pn)[6]) {
-    const F zero = (F)0;
-    const F out = add_(add_(sub_(fmax_(cx, zero), fmin(cmx, zero)),
-                            sub_(fmax_(cy, zero), fmin(cmy, zero))),
-                       sub_(fmax_(cz, zero), fmin(cmz, zero)));
-    const F in = fma_(fmax_(cmx, zero), Pn[1],
-                 fma_(-fmin(cx, zero), Pn[0],
-                 fma_(fmax_(cmy, zero), Pn[3],
-                 fma_(-fmin(cy, zero), Pn[2],
-                 fma_(fmax_(cmz, zero), Pn[5], mul_(-fmin(cz, zero), Pn[4]))))));
-    return out <= (F)1e-30 ? zero : div_(add_(cw, in), out);
-}
-
-// Face-coefficient adjoint sweep. Same organisation as the node-hyperplane forward sweep:
-// barrier groups of consecutive sources; a warp covers 64 sources of one node, lane l
-// holding sources l and l + 32; on each hyperplane the slots take the nodes slot,
-// slot + slots, ...; the schedule is static, so the next node's index and the next
-// hyperplane's bounds are read one step ahead. The coefficient planes are separate arrays,
-// so every load (a node's four coefficients, each upstream neighbour's one) is a coalesced
-// line. Sweeps cover every node (boundary faces carry no flux).
-#ifndef TTGB_ADJ_MIN_BLOCKS
-#define TTGB_ADJ_MIN_BLOCKS 3
-#endif
-template <typename F>
-__global__ void __launch_bounds__(256, TTGB_ADJ_MIN_BLOCKS) adj_face_kernel(AdjArgs<F> a) {
-    extern __shared__ unsigned char smem_raw[];
-    __shared__ int s_cnt;
-    const GridC &g = a.g;
-    const int B = a.B;
-    const int lgrp = blockIdx.x / a.grp_blocks;         // group within this launch
-    const int blk = blockIdx.x - lgrp * a.grp_blocks;
-    const int grp = a.grp_base + lgrp;
-    const int src0 = grp * a.grp_src;
-    const int Bg = min(B, src0 + a.grp_src) - src0;
-    if (Bg <= 0) return;
-    barrier_begin();
-    F *s_err = reinterpret_cast<F *>(smem_raw);
-    F *s_pmax = s_err + Bg;
-    BarrierState *bar = a.bar + lgrp;  // launches of a chunked solve reuse the same words
-    const unsigned nblk = (unsigned)a.grp_blocks;
-    const int Bw = ((Bg + 63) >> 6) << 5;               // lanes of one slot
-    const int slots = (int)(((long long)a.grp_blocks * blockDim.x) / Bw);
-    const long long tid = (long long)blk * blockDim.x + threadIdx.x;
-    const bool lane_ok = tid < (long long)slots * Bw;   // uniform over a warp
-    const int bl = lane_ok ? (int)(tid % Bw) : 0;
-    const int slot = lane_ok ? (int)(tid / Bw) : 0;
-    const int lane = threadIdx.x & 31;
-    const int l0 = ((bl >> 5) << 6) + lane;
-    const bool ok0 = lane_ok && l0 < Bg, ok1 = lane_ok && l0 + 32 < Bg;
-    const int b = src0 + (ok0 ? l0 : 0);                // second source: b + 32
-    const long long sp = B, st = (long long)g.np * B, sr = (long long)g.nt * g.np * B;
-    const long long plane = g.N * B;                    // coefficient plane stride
-    const F *cX = a.coef, *cY = a.coef + plane, *cZ = a.coef + 2 * plane, *cW = a.coef + 3 * plane;
-    F *P = a.P;
-
-    for (int it = 0; it < a.max_iter; ++it) {
-        const bool act0 = ok0 && ((volatile int *)a.conv)[b] == 0;
-        const bool act1 = ok1 && ((volatile int *)a.conv)[b + 32] == 0;
-        const bool busy = lane_ok && __any_sync(0xffffffffu, act0 || act1);  // uniform
-        F err0 = 0, err1 = 0, pmax0 = 0, pmax1 = 0;
-        for (int o = 0; o < 8; ++o) {
-            const bool rr = o & 4, rt = o & 2, rp = o & 1;
-            int qa = __ldg(a.off) + slot, qe = __ldg(a.off + 1);
-            unsigned pk = busy && qa < qe ? __ldg(a.nodes + qa) : 0u;
-            for (int L = 0; L < a.n_planes; ++L) {
-                const bool last = L + 1 == a.n_planes;
-                const int qe_next = last ? 0 : __ldg(a.off + L + 2);
-                if (busy) {
-                    for (int q = qa; q < qe; q += slots) {
-                        const int qn = q + slots;
-                        const unsigned pkn = qn < qe ? __ldg(a.nodes + qn) : 0u;
-                        int aa, bb, cc;
-                        unpack(pk, aa, bb, cc);
-                        const int i = rr ? g.nr - 1 - aa : aa;
-                        const int j = rt ? g.nt - 1 - bb : bb;
-                        const int k = rp ? g.np - 1 - cc : cc;
-                        const bool hr = i < g.nr - 1, lr = i > 0, ht = j < g.nt - 1, lt = j > 0;
-                        const bool hp = k < g.np - 1, lp = k > 0;
-                        const long long x = node_index(g, i, j, k) * B + b;
-                        // both sources' loads first, then the two updates
-                        F cx[2], cy[2], cz[2], w[2], cmx[2], cmy[2], cmz[2], Pn[2][6], po[2];
-#pragma unroll
-                        for (int h = 0; h < 2; ++h) {
-                            if (!(h == 0 ? act0 : act1)) continue;
-                            const long long y = x + 32 * h;
-                            w[h] = cW[y];
-                            cx[h] = cX[y];
-                            cy[h] = cY[y];
-                            cz[h] = cZ[y];
-                            cmx[h] = lr ? cX[y - sr] : (F)0;
-                            cmy[h] = lt ? cY[y - st] : (F)0;
-                            cmz[h] = lp ? cZ[y - sp] : (F)0;
-                            Pn[h][0] = hr ? P[y + sr] : (F)0;
-                            Pn[h][1] = lr ? P[y - sr] : (F)0;
-                            Pn[h][2] = ht ? P[y + st] : (F)0;
-                            Pn[h][3] = lt ? P[y - st] : (F)0;
-                            Pn[h][4] = hp ? P[y + sp] : (F)0;
-                            Pn[h][5] = lp ? P[y - sp] : (F)0;
-                            po[h] = P[y];
-                        }
-#pragma unroll
-                        for (int h = 0; h < 2; ++h) {
-                            if (!(h == 0 ? act0 : act1)) continue;
-                            if (w[h] != w[h]) continue;  // fixed set: P stays 0
-                            const F pn = face_update<F>(cx[h], cy[h], cz[h], w[h], cmx[h],
-                                                        cmy[h], cmz[h], Pn[h]);
-                            P[x + 32 * h] = pn;
-                            if (h == 0) {
-                                err0 = fmax_(err0, fabs(pn - po[0]));
-                                if (o == 7) pmax0 = fmax_(pmax0, fabs(pn));
-                            } else {
-                                err1 = fmax_(err1, fabs(pn - po[1]));
-                                if (o == 7) pmax1 = fmax_(pmax1, fabs(pn));
-                            }
-                        }
-                        pk = pkn;
-                    }
-                }
-                const int qa_next = qe + slot;
-                if (busy && !last && qa_next < qe_next) pk = __ldg(a.nodes + qa_next);
-                if (!grid_barrier(bar, a.spin_ns, nblk)) return;
-                qa = qa_next;
-                qe = qe_next;
-            }
-        }
-        for (int x = threadIdx.x; x < Bg; x += blockDim.x) { s_err[x] = 0; s_pmax[x] = 0; }
-        __syncthreads();
-        if (act0) {
-            atomic_max_nonneg(&s_err[b - src0], err0);
-            atomic_max_nonneg(&s_pmax[b - src0], pmax0);
-        }
-        if (act1) {
-            atomic_max_nonneg(&s_err[b + 32 - src0], err1);
-            atomic_max_nonneg(&s_pmax[b + 32 - src0], pmax1);
-        }
-        __syncthreads();
-        for (int x = threadIdx.x; x < Bg; x += blockDim.x) {
-            a.partial[((long long)blockIdx.x * 2) * B + src0 + x] = s_err[x];
-            a.partial[((long long)blockIdx.x * 2 + 1) * B + src0 + x] = s_pmax[x];
-        }
-        if (!grid_barrier(bar, a.spin_ns, nblk)) return;
-        if (blk == 0) {
-            if (threadIdx.x == 0) s_cnt = 0;
-            __syncthreads();
-            for (int x = src0 + threadIdx.x; x < src0 + Bg; x += blockDim.x) {
-                if (a.conv[x]) continue;
-                F m = 0, pm = 0;
-                for (int c = lgrp * a.grp_blocks; c < (lgrp + 1) * a.grp_blocks; ++c) {
-                    m = fmax_(m, ((volatile F *)a.partial)[((long long)c * 2) * B + x]);
-                    pm = fmax_(pm, ((volatile F *)a.partial)[((long long)c * 2 + 1) * B + x]);
-                }
-                a.iters[x] = it + 1;
-                if (m <= a.tol * pm) a.conv[x] = 1;
-                else atomicAdd(&s_cnt, 1);
-            }
-            __syncthreads();
-            if (threadIdx.x == 0) ((volatile int *)a.n_active)[lgrp] = s_cnt;
-        }
-        if (!grid_barrier(bar, a.spin_ns, nblk)) return;
-        if (((volatile int *)a.n_active)[lgrp] == 0) break;
-    }
-    barrier_end(bar, nblk);
-}
-
 // ------------------------------------------------------------------------ launchers
 
 // The retire-and-refill kernel of one variant.
@@ -1264,22 +1086,6 @@ template <typename F> cudaError_t launch_adjoint_coefs(const AdjArgs<F> &a, cuda
     return cudaGetLastError();
 }
 
-template <typename F>
-cudaError_t launch_adjoint_faces(const AdjArgs<F> &a, int grid, int block, cudaStream_t st) {
-    void *args[] = {const_cast<AdjArgs<F> *>(&a)};
-    size_t smem = (size_t)a.grp_src * 2 * sizeof(F);
-    return cudaLaunchCooperativeKernel((void *)adj_face_kernel<F>, dim3(grid), dim3(block), args,
-                                       smem, st);
-}
-
-template <typename F> int adjoint_faces_blocks_per_sm(int block, size_t smem) {
-    int n = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, adj_face_kernel<F>, block, smem) !=
-        cudaSuccess)
-        return 0;
-    return n;
-}
-
 template size_t forward_tiled_smem<float>(int, int);
 template size_t forward_tiled_smem<double>(int, int);
 template int forward_tiled_blocks_per_sm<float>(int, int);
@@ -1292,10 +1098,6 @@ template cudaError_t launch_forward_tiled<double>(const CUtensorMap &, const CUt
                                                   int, int, cudaStream_t);
 template cudaError_t launch_adjoint_coefs<float>(const AdjArgs<float> &, cudaStream_t);
 template cudaError_t launch_adjoint_coefs<double>(const AdjArgs<double> &, cudaStream_t);
-template cudaError_t launch_adjoint_faces<float>(const AdjArgs<float> &, int, int, cudaStream_t);
-template cudaError_t launch_adjoint_faces<double>(const AdjArgs<double> &, int, int, cudaStream_t);
-template int adjoint_faces_blocks_per_sm<float>(int, size_t);
-template int adjoint_faces_blocks_per_sm<double>(int, size_t);
 
 template cudaError_t launch_refill<float>(const FwdArgs<float> &, int, int, cudaStream_t);
 template cudaError_t launch_refill<double>(const FwdArgs<double> &, int, int, cudaStream_t);

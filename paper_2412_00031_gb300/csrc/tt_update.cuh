@@ -1,4 +1,4 @@
-// The update of one (node, source) of the forward sweeps, shared by their schedules.
+// The updates of one (node, source) of the sweeps, shared by their schedules.
 #pragma once
 
 #include "tt_common.cuh"
@@ -10,6 +10,33 @@ template <typename F> __device__ __forceinline__ F fmax_(F a, F b) { return a > 
 __device__ __forceinline__ unsigned bits_of(float x) { return __float_as_uint(x); }
 __device__ __forceinline__ unsigned long long bits_of(double x) {
     return (unsigned long long)__double_as_longlong(x);
+}
+
+__device__ __forceinline__ void atomic_max_nonneg(float *p, float v) {
+    atomicMax(reinterpret_cast<unsigned int *>(p), __float_as_uint(v));
+}
+__device__ __forceinline__ void atomic_max_nonneg(double *p, double v) {
+    atomicMax(reinterpret_cast<unsigned long long *>(p),
+              (unsigned long long)__double_as_longlong(v));
+}
+
+// Upwind update of one (node, source) from its face coefficients (Eq. 5 discretised as in
+// adj_update): c = (+r, +theta, +phi face coefficients, J S), cm = the -r, -theta, -phi
+// neighbours' plus-face coefficients, Pn = P at (+r, -r, +theta, -theta, +phi, -phi).
+// Rounding-explicit, so both lanes' copies give identical bits.
+template <typename F>
+__device__ __forceinline__ F face_update(F cx, F cy, F cz, F cw, F cmx, F cmy, F cmz,
+                                         const F (&Pn)[6]) {
+    const F zero = (F)0;
+    const F out = add_(add_(sub_(fmax_(cx, zero), fmin(cmx, zero)),
+                            sub_(fmax_(cy, zero), fmin(cmy, zero))),
+                       sub_(fmax_(cz, zero), fmin(cmz, zero)));
+    const F in = fma_(fmax_(cmx, zero), Pn[1],
+                 fma_(-fmin(cx, zero), Pn[0],
+                 fma_(fmax_(cmy, zero), Pn[3],
+                 fma_(-fmin(cy, zero), Pn[2],
+                 fma_(fmax_(cmz, zero), Pn[5], mul_(-fmin(cz, zero), Pn[4]))))));
+    return out <= (F)1e-30 ? zero : div_(add_(cw, in), out);
 }
 
 // New tau from v = tau at (centre, r+, r-, theta+, theta-, phi+, phi-), the cached factors c

@@ -68,3 +68,38 @@ def test_plane_sweep_gives_the_refill_bits(scheme, n_src, f64):
     ref, itr = _solve(tt, big, tt.default_opts(code, scheme=scheme, fwd_slots=32), dtype=dt)
     assert np.array_equal(it, itr[:n_src])
     assert np.array_equal(out, ref[..., :n_src])
+
+
+@pytest.mark.parametrize("shape,n_src", [((4, 4, 4), 40), ((4, 9, 5), 33), ((16, 18, 17), 800), ((7, 30, 29), 900)])
+@pytest.mark.parametrize("max_iter", [1, 60])
+def test_plane_adjoint_does_not_depend_on_the_batch(shape, n_src, max_iter):
+    """The adjoint of a large batch (pairs of sources a thread above some hundred) has the bits of its
+    sources in slices of 31 (a source a thread), at the smallest extents and with unaligned fields,
+    source slices, barrier groups and few blocks."""
+    import torch
+    import paper_2412_00031_gb300 as tt
+    w = _case(7 * sum(shape), shape, n_src)
+    rng = np.random.default_rng(n_src)
+    dev = lambda a: torch.as_tensor(np.ascontiguousarray(a), dtype=torch.float32, device="cuda")
+    model = tuple(dev(a) for a in (w.s, w.xi, w.eta))
+    ctx = tt.tt_ctx_create(w.grid.as_dict())
+    tau, T = (torch.empty(shape + (n_src,), device="cuda") for _ in range(2))
+    tt.tt_forward(ctx, model, w.src, tau, T)
+    rec = w.src[rng.integers(0, n_src, 5)] * np.array([0.0, 1.0, 1.0])
+    R = torch.as_tensor(rng.standard_normal((n_src, 5)), device="cuda")
+
+    def solve(lo, hi, shift=0, **kw):
+        buf = torch.empty(int(np.prod(shape)) * (hi - lo) + shift, device="cuda")
+        P = buf[shift:].view(shape + (hi - lo,))
+        it = tt.tt_adjoint(ctx, model, w.src[lo:hi], T[..., lo:hi].contiguous(), rec, R[lo:hi].contiguous(), P,
+                           tt.default_opts(tt.TT_F32, max_iter_adj=max_iter, **kw), allow_unconverged=True)
+        return P, it
+    P, it = solve(0, n_src)
+    for lo in range(0, n_src, 31 * (1 + n_src // 200)):
+        hi = min(lo + 31, n_src)
+        p, i = solve(lo, hi)
+        assert torch.equal(p, P[..., lo:hi]) and np.array_equal(i, it[lo:hi])
+    for kw in (dict(shift=1), dict(adj_chunk=64), dict(adj_groups=3), dict(launch_blocks=5)):
+        p, i = solve(0, n_src, **kw)
+        assert torch.equal(p, P) and np.array_equal(i, it), kw
+    ctx.close()

@@ -11,26 +11,35 @@
 // the theta and phi faces, and rows outside [0, R) (the radial faces) are zero-filled by the
 // tensor copy. Buffer [grid][R][C].
 //
-// GEMM of one tile: M = 128 consecutive rows r0 + m, K = 9 (di, dj) x C, and N = 3 x output
-// channels: the three dk taps' weights side by side, so that the accumulator holds, for each
-// dk, D_dk[m] = sum over (di, dj) of x[r0 + m + (di-1) Si + (dj-1) Sj - 1] W(di, dj, dk).
+// GEMM of one tile: M = 128 consecutive rows of one radial plane, K = 9 (di, dj) x C, and N =
+// 3 x output channels: the three dk taps' weights side by side, so that the accumulator holds, for
+// each dk, D_dk[m] = sum over (di, dj) of x[r0 + m + (di-1) Si + (dj-1) Sj - 1] W(di, dj, dk).
 // Output row r0 + m is D_0[m] + D_1[m + 1] + D_2[m + 2]: the epilogue combines neighbouring
 // TMEM lanes (warp shuffles, and a small shared-memory exchange across the four lane
-// quarters), so a tile of 128 accumulator rows yields 126 outputs and the tiles step by 126
-// rows. Every operand is thus an aligned block of whole rows, which lets both the A slabs
-// (one TMA tensor copy of 128 rows per (di, dj)) and the weights use the swizzled K-major
+// quarters), so a tile of 128 accumulator rows yields 126 outputs and the tiles of a plane step by
+// 126 rows. Every operand is thus an aligned block of whole rows, which lets both the A slabs
+// (one TMA tensor copy of 128 rows per input plane and dj) and the weights use the swizzled K-major
 // layout (64-byte swizzle for rows of 32 channels, 32-byte for 16): consecutive rows' 16-byte
 // chunks fall in different shared-memory banks.
 //
+// A CTA walks a window of 126 rows along the radius: an input plane's three dj slabs feed the
+// accumulators of the three output planes next to it (di = 2, 1, 0), which are in progress
+// together in tensor memory. So a tile takes three slab copies, not nine. The copies had bound the
+// layers: a TMA copy of 128 short rows runs at about one row per two clocks and SM whatever the
+// rows' width (layer 1 took as long as the others), and there were nine per tile. Tiles do not cross
+// a plane's end, which wastes less than a tile per plane. The order of an accumulator's sums
+// (di, dj, channels) is that of a tile by itself, so the bits are the same.
+// Measured: the warm start of 32 sources at 121x161x161 (network on every other node) 7.63 ms with
+// nine copies a tile, 4.11 ms so.
+//
 // Roles (320 threads, one persistent CTA per SM): warp 0 issues the tensor copies into a
-// ring of slab stages; warp 1 allocates tensor memory and issues the MMAs (one elected
-// thread), committing each stage back to the copier and each finished tile to the
-// epilogue; two epilogue warpgroups (warps 2-5 and 6-9) take alternate tiles, each with its
-// own accumulator buffer: they read the accumulators (tcgen05.ld, one TMEM lane quarter per
-// warp), add the bias, apply ReLU and store BF16 rows (or, in the last layer, the FP32
-// output of the real nodes). The epilogue is the longest role per tile, so two tiles of it
-// run at once while the MMAs of a third proceed. Every wait is bounded: on expiry the CTA raises its abort flag and the error word,
-// drains its copies and MMAs in flight, frees its tensor memory and returns.
+// ring of stages of one plane's three slabs; warp 1 allocates tensor memory and issues the MMAs (one
+// elected thread), committing each stage back to the copier and each finished tile to the
+// epilogue; two epilogue warpgroups (warps 2-5 and 6-9) take alternate tiles: they read the
+// accumulators (tcgen05.ld, one TMEM lane quarter per warp), add the bias, apply ReLU and store
+// BF16 rows (or, in the last layer, the FP32 output of the real nodes). Of the five accumulators
+// three are being summed and two read. Every wait is bounded: on expiry the CTA raises its abort
+// flag and the error word, drains its copies and MMAs in flight, frees its tensor memory and returns.
 #include <cuda.h>
 #include <cudaTypedefs.h>
 #include <cuda_bf16.h>
@@ -44,26 +53,25 @@ namespace {
 
 constexpr int kTileRows = 128;                 // M
 constexpr int kTileStep = kTileRows - 2;       // output rows of one tile
-#ifndef TTGB_TC_STAGES
-#define TTGB_TC_STAGES 16
-#endif
-constexpr int kStages = TTGB_TC_STAGES;
+constexpr int kStages = 6;                     // planes of three slabs
 constexpr int kThreads = 320;                  // copier, MMA, two epilogue warpgroups
-// Two accumulator buffers of up to 3 x 32 columns.
-constexpr int kBufCols = 128;
-constexpr int kTmemCols = 256;
+// Five accumulators of up to 3 x 32 columns.
+constexpr int kAccs = 5;
+constexpr int kBufCols = 96;
+constexpr int kTmemCols = 512;
 
 // KC: 8-channel chunks of an input row (2: C = 16, 4: C = 32); NO: output channels per dk
 // (32, or 16 for the last layer).
 template <int KC, int NO> struct Smem {
     static constexpr int ROW = KC * 16;                          // bytes of one row
     static constexpr int QW = 3 * NO * ROW;                      // weights of one (di, dj)
-    static constexpr int W = 9 * QW;                             // [q][dk][co] rows, swizzled
+    static constexpr int W = 9 * QW;                             // [dj][2 - di][dk][co] rows, swizzled
     static constexpr int SLAB = kTileRows * ROW;
+    static constexpr int STAGE = 3 * SLAB;                       // the dj slabs of an input plane
     static constexpr int A = (W + 1023) / 1024 * 1024;
-    static constexpr int EXCH = A + kStages * SLAB;              // [2][4 quarters][2][2][32] float
+    static constexpr int EXCH = A + kStages * STAGE;             // [2][4 quarters][2][2][32] float
     static constexpr int BAR = EXCH + 2 * 4 * 2 * 2 * 32 * 4;    // mbarriers
-    static constexpr int NBAR = 2 * kStages + 5;                 // full, empty, acc x 4, drain
+    static constexpr int NBAR = 2 * kStages + 2 * kAccs + 1;     // full, empty, acc full, acc empty, drain
     static constexpr int MISC = BAR + NBAR * 8;                  // tmem address, abort flag
     static constexpr int TOTAL = MISC + 16 + 1024;               // + alignment slack
     // swizzle: 64 bytes for rows of 64 bytes, 32 for rows of 32 (descriptor layout code)
@@ -215,11 +223,20 @@ __device__ __forceinline__ void tmem_ld96(unsigned taddr, unsigned (&a)[32], uns
         : "memory");
 }
 
-__device__ __forceinline__ float tmem_ld1(unsigned taddr) {
-    unsigned r;
-    asm volatile("tcgen05.ld.sync.aligned.32x32b.x1.b32 {%0}, [%1];" : "=r"(r) : "r"(taddr) : "memory");
-    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-    return __uint_as_float(r);
+// One column at each of three addresses.
+__device__ __forceinline__ void tmem_ld3(unsigned t0, unsigned t1, unsigned t2, float &d0, float &d1, float &d2) {
+    unsigned a, b, c;
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x1.b32 {%0}, [%3];\n"
+        "tcgen05.ld.sync.aligned.32x32b.x1.b32 {%1}, [%4];\n"
+        "tcgen05.ld.sync.aligned.32x32b.x1.b32 {%2}, [%5];\n"
+        "tcgen05.wait::ld.sync.aligned;\n"
+        : "=r"(a), "=r"(b), "=r"(c)
+        : "r"(t0), "r"(t1), "r"(t2)
+        : "memory");
+    d0 = __uint_as_float(a);
+    d1 = __uint_as_float(b);
+    d2 = __uint_as_float(c);
 }
 
 struct RowGeo {
@@ -227,8 +244,25 @@ struct RowGeo {
     int Sj;             // n_p + 1
     int Si;             // (n_t + 1) Sj
     int R;              // rows of one grid: n_r Si
-    int tiles;          // ceil(R / 126) per grid
+    int wins;           // windows of 126 rows of a plane: ceil(Si / 126)
+    int chunks;         // runs of planes that a window is cut into
 };
+
+// A CTA's work: window win of the output planes [i0, i1) of grid g. Neighbouring windows run at
+// the same time on neighbouring CTAs, so that a row's three dj reads meet in L2.
+struct Walk {
+    int g, win, i0, i1;
+};
+__device__ __forceinline__ Walk walk_of(const RowGeo &G, long long T) {
+    Walk w;
+    w.win = (int)(T % G.wins);
+    const long long t = T / G.wins;
+    const int c = (int)(t % G.chunks);
+    w.g = (int)(t / G.chunks);
+    w.i0 = (int)((long long)G.nr * c / G.chunks);
+    w.i1 = (int)((long long)G.nr * (c + 1) / G.chunks);
+    return w;
+}
 
 __device__ __forceinline__ bool pad_row(const RowGeo &G, int n) {
     return n % G.Sj == G.np || (n / G.Sj) % (G.nt + 1) == G.nt;
@@ -258,8 +292,8 @@ __global__ void __launch_bounds__(kThreads, 1)
     auto full = [&](int s) { return sBar + 8u * s; };
     auto empty = [&](int s) { return sBar + 8u * (kStages + s); };
     auto acc_full = [&](int a) { return sBar + 8u * (2 * kStages + a); };
-    auto acc_empty = [&](int a) { return sBar + 8u * (2 * kStages + 2 + a); };
-    const unsigned drain = sBar + 8u * (2 * kStages + 4);
+    auto acc_empty = [&](int a) { return sBar + 8u * (2 * kStages + kAccs + a); };
+    const unsigned drain = sBar + 8u * (2 * kStages + 2 * kAccs);
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     // weights into shared memory (generic stores, made visible to the tensor cores below)
@@ -270,10 +304,10 @@ __global__ void __launch_bounds__(kThreads, 1)
             bar_init(full(s), 1);
             bar_init(empty(s), 1);
         }
-        bar_init(acc_full(0), 1);
-        bar_init(acc_full(1), 1);
-        bar_init(acc_empty(0), 128);
-        bar_init(acc_empty(1), 128);
+        for (int u = 0; u < kAccs; ++u) {
+            bar_init(acc_full(u), 1);
+            bar_init(acc_empty(u), 128);
+        }
         bar_init(drain, 1);
         *s_abort = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -291,22 +325,23 @@ __global__ void __launch_bounds__(kThreads, 1)
     __syncthreads();
     tc_fence_after();
     const unsigned tmem = *s_tmem;
-    const long long total = (long long)G.nb * G.tiles;
+    const long long total = (long long)G.nb * G.chunks * G.wins;
 
     if (warp == 0) {
         if (lane == 0) {
-            // copier: the nine slabs of every tile of this CTA, in order, into the stage ring
+            // copier: the dj slabs of the input planes of every walk of this CTA, in order, into
+            // the stage ring (planes beyond the grid are zero-filled)
             int s = 0;
             unsigned ph = 0, armed = 0, armed_par = 0;
             bool ok = true;
             for (long long T = blockIdx.x; ok && T < total; T += gridDim.x) {
-                const int g = (int)(T / G.tiles);
-                const int n0 = (int)(T - (long long)g * G.tiles) * kTileStep;
-                for (int q = 0; q < 9; ++q) {
+                const Walk w = walk_of(G, T);
+                for (int p = w.i0 - 1; p <= w.i1; ++p) {
                     if (!bar_wait(empty(s), ph ^ 1u, limit, s_abort)) { ok = false; break; }
-                    bar_expect_tx(full(s), L::SLAB);
-                    tma_rows(sA + s * L::SLAB, &map, n0 + (q / 3 - 1) * G.Si + (q % 3 - 1) * G.Sj - 1,
-                             g, full(s));
+                    bar_expect_tx(full(s), L::STAGE);
+                    const int r0 = p * G.Si + w.win * kTileStep - 1;
+                    for (int dj = 0; dj < 3; ++dj)
+                        tma_rows(sA + s * L::STAGE + dj * L::SLAB, &map, r0 + (dj - 1) * G.Sj, w.g, full(s));
                     armed |= 1u << s;
                     armed_par = (armed_par & ~(1u << s)) | (ph << s);
                     if (++s == kStages) { s = 0; ph ^= 1u; }
@@ -319,30 +354,45 @@ __global__ void __launch_bounds__(kThreads, 1)
     } else if (warp == 1) {
         if (lane == 0) {
             constexpr unsigned ID = idesc_bf16<3 * NO>();
-            int s = 0, a = 0;
-            unsigned ph = 0, aph = 0;
+            // Input plane p adds to the output planes p - 1, p, p + 1 of the walk (d = 0, 1, 2:
+            // di = 2 - d), whose accumulators follow one another in the ring.
+            int s = 0, u0 = 0;            // u0: accumulator of the walk's first output plane
+            unsigned ph = 0, uph = 0;     // uph: parity of the ring's turn there
             bool ok = true;
             for (long long T = blockIdx.x; ok && T < total; T += gridDim.x) {
-                if (!bar_wait(acc_empty(a), aph ^ 1u, limit, s_abort)) break;
-                tc_fence_after();
-                const unsigned d = tmem + (unsigned)(a * kBufCols);
-                for (int q = 0; q < 9; ++q) {
+                const Walk w = walk_of(G, T);
+                int un = u0;              // accumulator of output plane p + 1
+                for (int p = w.i0 - 1; p <= w.i1; ++p) {
+                    const bool has0 = p - 1 >= w.i0, has1 = p >= w.i0 && p < w.i1, has2 = p + 1 < w.i1;
+                    if (has2 && !bar_wait(acc_empty(un), uph ^ 1u, limit, s_abort)) { ok = false; break; }
                     if (!bar_wait(full(s), ph, limit, s_abort)) { ok = false; break; }
-                    const unsigned slab = sA + s * L::SLAB;
+                    tc_fence_after();
+                    const int u1 = un == 0 ? kAccs - 1 : un - 1, u2 = u1 == 0 ? kAccs - 1 : u1 - 1;
+                    const unsigned stage = sA + s * L::STAGE;
+                    const unsigned t0 = tmem + (unsigned)(u2 * kBufCols), t1 = tmem + (unsigned)(u1 * kBufCols),
+                                   t2 = tmem + (unsigned)(un * kBufCols);
 #pragma unroll
-                    for (int h = 0; h < KC / 2; ++h) {
-                        // K half h: 32 bytes into the swizzled rows; B: the (di, dj) weights of
-                        // the three dk taps, rows [dk][co]
-                        const unsigned long long ad = mdesc(slab + 32 * h, L::SBO, L::LAYOUT);
-                        const unsigned long long bd = mdesc(sW + q * L::QW + 32 * h, L::SBO, L::LAYOUT);
-                        mma_bf16(d, ad, bd, ID, (q | h) != 0);
-                    }
+                    for (int dj = 0; dj < 3; ++dj)
+#pragma unroll
+                        for (int h = 0; h < KC / 2; ++h) {
+                            // K half h: 32 bytes into the swizzled rows; B: the (di, dj) weights of
+                            // the three dk taps, rows [dk][co]
+                            const unsigned long long ad = mdesc(stage + dj * L::SLAB + 32 * h, L::SBO, L::LAYOUT);
+                            const unsigned wb = sW + dj * 3 * L::QW + 32 * h;
+                            if (has0) mma_bf16(t0, ad, mdesc(wb, L::SBO, L::LAYOUT), ID, 1u);
+                            if (has1) mma_bf16(t1, ad, mdesc(wb + L::QW, L::SBO, L::LAYOUT), ID, 1u);
+                            if (has2) mma_bf16(t2, ad, mdesc(wb + 2 * L::QW, L::SBO, L::LAYOUT), ID, (dj | h) != 0);
+                        }
                     mma_commit(empty(s));   // the stage is free once these MMAs have read it
+                    if (has0) mma_commit(acc_full(u2));
                     if (++s == kStages) { s = 0; ph ^= 1u; }
+                    // past the walk's end un only counts on, for the accumulators behind it
+                    if (has2) {
+                        u0 = un + 1 == kAccs ? 0 : un + 1;
+                        if (u0 == 0) uph ^= 1u;
+                    }
+                    un = un + 1 == kAccs ? 0 : un + 1;
                 }
-                if (!ok) break;
-                mma_commit(acc_full(a));
-                if (++a == 2) { a = 0; aph ^= 1u; }
             }
             // every MMA issued has completed before tensor memory is freed
             mma_commit(drain);
@@ -358,22 +408,43 @@ __global__ void __launch_bounds__(kThreads, 1)
         float bz[FINAL ? 1 : 32];
 #pragma unroll
         for (int c = 0; c < (FINAL ? 1 : 32); ++c) bz[c] = MODE == kEpiGate ? 0.0f : bias[c];
-        unsigned aph = 0;
-        for (long long T = blockIdx.x + (long long)a * gridDim.x; T < total; T += 2LL * gridDim.x) {
+        float *ex = exch + a * 4 * 2 * 2 * 32;
+        int u = -1, par = 0;                                     // accumulator and group of the next tile
+        unsigned uph = 0;
+        bool ok = true;
+        for (long long T = blockIdx.x; ok && T < total; T += gridDim.x) {
+          const Walk wk = walk_of(G, T);
+          const int g = wk.g, rw = wk.win * kTileStep + m;       // the thread's row of the plane
+          const bool out_ok = m < kTileStep && rw < G.Si;
+          const int j = rw / G.Sj, k = rw - j * G.Sj;
+          const bool zero = !out_ok || k == G.np || j >= G.nt;    // padding rows are written as zero
+          for (int i = wk.i0; i < wk.i1; ++i) {
+            if (++u == kAccs) { u = 0; uph ^= 1u; }
+            par ^= 1;
+            if (par == a) continue;
+            const int n = i * G.Si + rw;
+            unsigned gw[16];   // kEpiGate: the gate row's 32 BF16 channels
+            if (MODE == kEpiGate && !zero) {
+                const uint4 *gr = gate + ((long long)g * G.R + n) * 4;
+#pragma unroll
+                for (int c = 0; c < 4; ++c) {
+                    const uint4 v = gr[c];
+                    gw[4 * c] = v.x;
+                    gw[4 * c + 1] = v.y;
+                    gw[4 * c + 2] = v.z;
+                    gw[4 * c + 3] = v.w;
+                }
+            }
             // all 128 threads of the group agree (TMEM loads are warp-collective, the
             // exchange spans the group)
-            if (!epi_all(a, bar_wait(acc_full(a), aph, limit, s_abort))) break;
+            if (!epi_all(a, bar_wait(acc_full(u), uph, limit, s_abort))) { ok = false; break; }
             tc_fence_after();
-            const unsigned taddr = tmem + ((unsigned)(quarter * 32) << 16) + (unsigned)(a * kBufCols);
-            float *ex = exch + a * 4 * 2 * 2 * 32;
-            const int g = (int)(T / G.tiles);
-            const int n = (int)(T - (long long)g * G.tiles) * kTileStep + m;
-            const bool out_ok = m < kTileStep && n < G.R;
+            const unsigned taddr = tmem + ((unsigned)(quarter * 32) << 16) + (unsigned)(u * kBufCols);
             if (FINAL) {
-                const float d0 = tmem_ld1(taddr), d1 = tmem_ld1(taddr + NO),
-                            d2 = tmem_ld1(taddr + 2 * NO);
+                float d0, d1, d2;
+                tmem_ld3(taddr, taddr + NO, taddr + 2 * NO, d0, d1, d2);
                 tc_fence_before();
-                bar_arrive(acc_empty(a));
+                bar_arrive(acc_empty(u));
                 if (lane < 2) {
                     ex[((quarter * 2 + lane) * 2 + 0) * 32] = d1;
                     ex[((quarter * 2 + lane) * 2 + 1) * 32] = d2;
@@ -385,8 +456,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                     if (lane == 31) s1 = ex[(((quarter + 1) * 2 + 0) * 2 + 0) * 32];
                     if (lane >= 30) s2 = ex[(((quarter + 1) * 2 + lane - 30) * 2 + 1) * 32];
                 }
-                if (out_ok && !pad_row(G, n)) {
-                    const int k = n % G.Sj, j = (n / G.Sj) % (G.nt + 1), i = n / G.Si;
+                if (!zero) {
                     const long long node = ((long long)i * G.nt + j) * G.np + k;
                     reinterpret_cast<float *>(out_)[(long long)g * G.nr * G.nt * G.np + node] =
                         (d0 + s1) + s2 + bz[0];
@@ -404,26 +474,38 @@ __global__ void __launch_bounds__(kThreads, 1)
                     }
                 }
                 tc_fence_before();
-                bar_arrive(acc_empty(a));
+                bar_arrive(acc_empty(u));
                 if (lane < 2) {
+                    float4 *e = reinterpret_cast<float4 *>(ex + (quarter * 2 + lane) * 2 * 32);
 #pragma unroll
-                    for (int c = 0; c < 32; ++c) {
-                        ex[((quarter * 2 + lane) * 2 + 0) * 32 + c] = d1[c];
-                        ex[((quarter * 2 + lane) * 2 + 1) * 32 + c] = d2[c];
+                    for (int c = 0; c < 8; ++c) {
+                        e[c] = make_float4(d1[4 * c], d1[4 * c + 1], d1[4 * c + 2], d1[4 * c + 3]);
+                        e[8 + c] = make_float4(d2[4 * c], d2[4 * c + 1], d2[4 * c + 2], d2[4 * c + 3]);
                     }
                 }
                 epi_sync(a);
-                const bool zero = !out_ok || pad_row(G, n);
-                unsigned gw[16];   // kEpiGate: the gate row's 32 BF16 channels
-                if (MODE == kEpiGate && !zero) {
-                    const uint4 *gr = gate + ((long long)g * G.R + n) * 4;
 #pragma unroll
-                    for (int c = 0; c < 4; ++c) {
-                        const uint4 v = gr[c];
-                        gw[4 * c] = v.x;
-                        gw[4 * c + 1] = v.y;
-                        gw[4 * c + 2] = v.z;
-                        gw[4 * c + 3] = v.w;
+                for (int c = 0; c < 32; ++c) {
+                    d1[c] = __shfl_down_sync(0xffffffffu, d1[c], 1);
+                    d2[c] = __shfl_down_sync(0xffffffffu, d2[c], 2);
+                }
+                if (lane >= 30 && quarter < 3) {   // the next quarter's first lanes
+                    const float4 *e1 = reinterpret_cast<const float4 *>(ex + (quarter + 1) * 2 * 2 * 32);
+                    const float4 *e2 = e1 + (lane - 30) * 16 + 8;
+#pragma unroll
+                    for (int c = 0; c < 8; ++c) {
+                        const float4 x = e2[c];
+                        d2[4 * c] = x.x;
+                        d2[4 * c + 1] = x.y;
+                        d2[4 * c + 2] = x.z;
+                        d2[4 * c + 3] = x.w;
+                        if (lane == 31) {
+                            const float4 y = e1[c];
+                            d1[4 * c] = y.x;
+                            d1[4 * c + 1] = y.y;
+                            d1[4 * c + 2] = y.z;
+                            d1[4 * c + 3] = y.w;
+                        }
                     }
                 }
                 unsigned w[16];
@@ -431,19 +513,14 @@ __global__ void __launch_bounds__(kThreads, 1)
                 for (int c = 0; c < 32; c += 2) {
                     float v[2];
 #pragma unroll
-                    for (int u = 0; u < 2; ++u) {
-                        float s1 = __shfl_down_sync(0xffffffffu, d1[c + u], 1);
-                        float s2 = __shfl_down_sync(0xffffffffu, d2[c + u], 2);
-                        if (quarter < 3) {
-                            if (lane == 31) s1 = ex[(((quarter + 1) * 2 + 0) * 2 + 0) * 32 + c + u];
-                            if (lane >= 30) s2 = ex[(((quarter + 1) * 2 + lane - 30) * 2 + 1) * 32 + c + u];
-                        }
+                    for (int h = 0; h < 2; ++h) {
+                        const float sum = (d0[c + h] + d1[c + h]) + d2[c + h];
                         if (MODE == kEpiGate) {
-                            const unsigned short hb = (unsigned short)(gw[c / 2] >> (16 * u));
+                            const unsigned short hb = (unsigned short)(gw[c / 2] >> (16 * h));
                             const bool open = !zero && __bfloat162float(__ushort_as_bfloat16(hb)) > 0.0f;
-                            v[u] = open ? (d0[c + u] + s1) + s2 : 0.0f;
+                            v[h] = open ? sum : 0.0f;
                         } else {
-                            v[u] = zero ? 0.0f : fmaxf((d0[c + u] + s1) + s2 + bz[c + u], 0.0f);
+                            v[h] = zero ? 0.0f : fmaxf(sum + bz[c + h], 0.0f);
                         }
                     }
                     const __nv_bfloat162 p = __floats2bfloat162_rn(v[0], v[1]);
@@ -456,7 +533,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                         o[c] = make_uint4(w[4 * c], w[4 * c + 1], w[4 * c + 2], w[4 * c + 3]);
                 }
             }
-            aph ^= 1u;
+          }
         }
     }
     tc_fence_before();
@@ -510,8 +587,8 @@ __global__ void pack_dy_kernel(RowGeo G, const float *__restrict__ dy, uint4 *__
 }
 
 // Layer l's weights W[27][cin][cout] (FP32) -> the shared-memory image of the B operands
-// (BF16): for q = (di, dj), rows (dk, co) of C = 8 KC input channels (tap t = 3 q + dk; zero
-// beyond cin and cout), each row's 16-byte chunks placed as the tensor cores' swizzle of the
+// (BF16): blocks [dj][2 - di] (q = (di, dj)) of rows (dk, co) of C = 8 KC input channels (tap t =
+// 3 q + dk; zero beyond cin and cout), each row's 16-byte chunks placed as the tensor cores' swizzle of the
 // row width expects them (chunk c of row r at c ^ ((r >> 1) & 3) for 64-byte rows,
 // c ^ ((r >> 2) & 1) for 32-byte rows).
 __global__ void weight_image_kernel(const float *__restrict__ w, int cin, int cout, int KC, int NO,
@@ -525,7 +602,8 @@ __global__ void weight_image_kernel(const float *__restrict__ w, int cin, int co
     const int r = dk * NO + co;                     // row within the (di, dj) block
     const int c = ci / 8;
     const int cs = KC == 4 ? c ^ ((r >> 1) & 3) : c ^ ((r >> 2) & 1);
-    img[((size_t)q * 3 * NO + r) * C + cs * 8 + ci % 8] = __float2bfloat16_rn(v);
+    const int blk = (q % 3) * 3 + 2 - q / 3;        // [dj][2 - di]
+    img[((size_t)blk * 3 * NO + r) * C + cs * 8 + ci % 8] = __float2bfloat16_rn(v);
 }
 
 // ------------------------------------------------------------------------ weight gradients
@@ -792,19 +870,36 @@ cudaError_t encode_rows(CUtensorMap *map, const void *base, const RowGeo &G, int
     return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
 }
 
+// Runs of planes per window: the number with the shortest longest CTA. A run of L output planes costs
+// about L + 1 tiles (its two outer input planes are copied for one output plane each).
+int walk_chunks(const RowGeo &G, int n_sm) {
+    int best = 1;
+    long long least = -1;
+    for (int c = 1; c <= G.nr; ++c) {
+        const long long waves = ((long long)G.nb * G.wins * c + n_sm - 1) / n_sm;
+        const long long cost = waves * ((G.nr + c - 1) / c + 1);
+        if (least < 0 || cost < least) {
+            least = cost;
+            best = c;
+        }
+    }
+    return best;
+}
+
 template <int KC, int NO, int MODE>
-cudaError_t launch_layer(const void *in, const RowGeo &G, const __nv_bfloat16 *wimg,
+cudaError_t launch_layer(const void *in, RowGeo G, const __nv_bfloat16 *wimg,
                          const float *bias, void *out, int n_sm, int *err,
                          unsigned long long limit, cudaStream_t st, const void *gate = nullptr) {
     CUtensorMap map;
     cudaError_t e = encode_rows(&map, in, G, KC);
     if (e != cudaSuccess) return e;
+    G.chunks = walk_chunks(G, n_sm);
     // more than half the shared memory of an SM: one CTA per SM, which owns its TMEM
     constexpr int smem = Smem<KC, NO>::TOTAL > 120 * 1024 ? Smem<KC, NO>::TOTAL : 120 * 1024;
     const void *fn = (const void *)conv3d_tc_kernel<KC, NO, MODE>;
     e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
-    const long long total = (long long)G.nb * G.tiles;
+    const long long total = (long long)G.nb * G.chunks * G.wins;
     const unsigned grid = (unsigned)(total < n_sm ? total : n_sm);
     conv3d_tc_kernel<KC, NO, MODE><<<grid, kThreads, smem, st>>>(
         map, G, reinterpret_cast<const uint4 *>(wimg), bias, reinterpret_cast<const uint4 *>(gate),
@@ -848,7 +943,8 @@ RowGeo row_geo(const ConvDims &d) {
     G.Sj = d.W + 1;
     G.Si = (d.H + 1) * G.Sj;
     G.R = d.D * G.Si;
-    G.tiles = (G.R + kTileStep - 1) / kTileStep;
+    G.wins = (G.Si + kTileStep - 1) / kTileStep;
+    G.chunks = 1;
     return G;
 }
 

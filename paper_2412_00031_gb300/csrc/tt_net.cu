@@ -302,34 +302,56 @@ __device__ __forceinline__ void net_axis_pos(int i, int c, int nc, int n, int &a
 }
 
 // tau = 1 + the trilinear interpolation of clamp(y) from the network grid (a NaN prediction
-// counts as 0), for the network-grid stride ng.c > 1.
+// counts as 0), for the network-grid stride ng.c > 1. A block takes up to 32 network cells along
+// phi and up to 32 sources: y is [source][node] and tau [node][source], so the cells' corners go
+// through shared memory, read along phi and used along the sources, once for the c x c x c nodes
+// of a cell. With a thread per (node, source) that gathered its eight corners from global memory,
+// a line each, the kernel was a third of a warm start: 32 sources at 121x161x161 (c = 2)
+// 1.20 ms, now 0.42 ms.
+constexpr int kUpCells = 32, kUpSrc = 32, kUpThreads = 256;
 template <typename F>
-__global__ void warm_tau_up_kernel(GridC g, NetGrid ng, int B, int b0, int nb,
-                                   const float *__restrict__ y, F *__restrict__ tau) {
-    const long long q = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (q >= g.N * nb) return;
-    const int bl = (int)(q % nb);
-    const long long n = q / nb;
-    const int k = (int)(n % g.np);
-    const long long tq = n / g.np;
-    const int j = (int)(tq % g.nt), i = (int)(tq / g.nt);
-    int a[3];
-    float f[3];
-    net_axis_pos(i, ng.c, ng.nr, g.nr, a[0], f[0]);
-    net_axis_pos(j, ng.c, ng.nt, g.nt, a[1], f[1]);
-    net_axis_pos(k, ng.c, ng.np, g.np, a[2], f[2]);
-    const float *yb = y + (long long)bl * ng.nr * ng.nt * ng.np;
-    float v = 0.0f;
-#pragma unroll
-    for (int u = 0; u < 8; ++u) {
-        const int di = u >> 2, dj = (u >> 1) & 1, dk = u & 1;
-        const float w = (di ? f[0] : 1.0f - f[0]) * (dj ? f[1] : 1.0f - f[1]) *
-                        (dk ? f[2] : 1.0f - f[2]);
-        const float yv = yb[((long long)(a[0] + di) * ng.nt + a[1] + dj) * ng.np + a[2] + dk];
-        const float c = yv == yv ? fminf(fmaxf(yv, kNetClampLo), kNetClampHi) : 0.0f;
-        v = fmaf(w, c, v);
+__global__ void __launch_bounds__(kUpThreads)
+    warm_tau_up_kernel(GridC g, NetGrid ng, int B, int b0, int nb, const float *__restrict__ y, F *__restrict__ tau) {
+    __shared__ float s_y[4][kUpCells + 1][kUpSrc + 1];
+    const int k_tiles = (ng.np - 2 + kUpCells) / kUpCells, s_tiles = (nb + kUpSrc - 1) / kUpSrc;
+    long long q = blockIdx.x;
+    const int s0 = (int)(q % s_tiles) * kUpSrc;
+    q /= s_tiles;
+    const int kc0 = (int)(q % k_tiles) * kUpCells;
+    q /= k_tiles;
+    const int jc = (int)(q % (ng.nt - 1)), ic = (int)(q / (ng.nt - 1));
+    const int ns = min(kUpSrc, nb - s0), cells = min(kUpCells, ng.np - 1 - kc0), kn = cells + 1;
+    for (int e = threadIdx.x; e < 4 * kn * ns; e += kUpThreads) {
+        const int kk = e % kn, r = e / kn, row = r & 3, b = r >> 2;
+        const float yv = y[(((long long)(s0 + b) * ng.nr + ic + (row >> 1)) * ng.nt + jc + (row & 1)) * ng.np + kc0 + kk];
+        s_y[row][kk][b] = yv == yv ? fminf(fmaxf(yv, kNetClampLo), kNetClampHi) : 0.0f;
     }
-    tau[n * B + b0 + bl] = (F)(1.0f + v);
+    __syncthreads();
+    // The cells' solver nodes: from the lower corner on, the axis's last node with its last cell. A
+    // thread keeps a (phi node, source)'s eight corners for all (r, theta) nodes of the cell.
+    const int i0 = ic * ng.c, j0 = jc * ng.c, k0 = kc0 * ng.c;
+    const int i1 = ic == ng.nr - 2 ? g.nr : i0 + ng.c, j1 = jc == ng.nt - 2 ? g.nt : j0 + ng.c;
+    const int k1 = kc0 + cells == ng.np - 1 ? g.np : (kc0 + cells) * ng.c;
+    const float li = (float)(min(i0 + ng.c, g.nr - 1) - i0), lj = (float)(min(j0 + ng.c, g.nt - 1) - j0);
+    for (int e = threadIdx.x; e < (k1 - k0) * ns; e += kUpThreads) {
+        const int k = k0 + e / ns, b = e % ns;
+        int ak;
+        float fk, c[8];
+        net_axis_pos(k, ng.c, ng.np, g.np, ak, fk);
+#pragma unroll
+        for (int u = 0; u < 8; ++u) c[u] = s_y[u >> 1][ak - kc0 + (u & 1)][b];
+        for (int i = i0; i < i1; ++i) {
+            const float fi = (float)(i - i0) / li;
+            for (int j = j0; j < j1; ++j) {
+                const float fj = (float)(j - j0) / lj;
+                float v = 0.0f;
+#pragma unroll
+                for (int u = 0; u < 8; ++u)
+                    v = fmaf((u & 4 ? fi : 1.0f - fi) * (u & 2 ? fj : 1.0f - fj) * (u & 1 ? fk : 1.0f - fk), c[u], v);
+                tau[node_index(g, i, j, k) * B + b0 + s0 + b] = (F)(1.0f + v);
+            }
+        }
+    }
 }
 
 __global__ void round_bf16_kernel(int n, const float *__restrict__ in, float *__restrict__ out) {
@@ -415,8 +437,11 @@ cudaError_t run_warm_tau(const GridC &g, const NetGrid &ng, int B, int b0, int n
                          const float *y, F *tau, cudaStream_t st) {
     if (ng.c == 1)
         warm_tau_kernel<F><<<blocks_of(g.N * nb, 256), 256, 0, st>>>(g.N, B, b0, nb, y, tau);
-    else
-        warm_tau_up_kernel<F><<<blocks_of(g.N * nb, 256), 256, 0, st>>>(g, ng, B, b0, nb, y, tau);
+    else {
+        const long long blocks = (long long)(ng.nr - 1) * (ng.nt - 1) * ((ng.np - 2 + kUpCells) / kUpCells) *
+                                 ((nb + kUpSrc - 1) / kUpSrc);
+        warm_tau_up_kernel<F><<<(unsigned)blocks, kUpThreads, 0, st>>>(g, ng, B, b0, nb, y, tau);
+    }
     return cudaGetLastError();
 }
 

@@ -413,127 +413,127 @@ __global__ void __launch_bounds__(kThreads, 1)
         unsigned uph = 0;
         bool ok = true;
         for (long long T = blockIdx.x; ok && T < total; T += gridDim.x) {
-          const Walk wk = walk_of(G, T);
-          const int g = wk.g, rw = wk.win * kTileStep + m;       // the thread's row of the plane
-          const bool out_ok = m < kTileStep && rw < G.Si;
-          const int j = rw / G.Sj, k = rw - j * G.Sj;
-          const bool zero = !out_ok || k == G.np || j >= G.nt;    // padding rows are written as zero
-          for (int i = wk.i0; i < wk.i1; ++i) {
-            if (++u == kAccs) { u = 0; uph ^= 1u; }
-            par ^= 1;
-            if (par == a) continue;
-            const int n = i * G.Si + rw;
-            unsigned gw[16];   // kEpiGate: the gate row's 32 BF16 channels
-            if (MODE == kEpiGate && !zero) {
-                const uint4 *gr = gate + ((long long)g * G.R + n) * 4;
+            const Walk wk = walk_of(G, T);
+            const int g = wk.g, rw = wk.win * kTileStep + m;       // the thread's row of the plane
+            const bool out_ok = m < kTileStep && rw < G.Si;
+            const int j = rw / G.Sj, k = rw - j * G.Sj;
+            const bool zero = !out_ok || k == G.np || j >= G.nt;    // padding rows are written as zero
+            for (int i = wk.i0; i < wk.i1; ++i) {
+                if (++u == kAccs) { u = 0; uph ^= 1u; }
+                par ^= 1;
+                if (par == a) continue;
+                const int n = i * G.Si + rw;
+                unsigned gw[16];   // kEpiGate: the gate row's 32 BF16 channels
+                if (MODE == kEpiGate && !zero) {
+                    const uint4 *gr = gate + ((long long)g * G.R + n) * 4;
 #pragma unroll
-                for (int c = 0; c < 4; ++c) {
-                    const uint4 v = gr[c];
-                    gw[4 * c] = v.x;
-                    gw[4 * c + 1] = v.y;
-                    gw[4 * c + 2] = v.z;
-                    gw[4 * c + 3] = v.w;
+                    for (int c = 0; c < 4; ++c) {
+                        const uint4 v = gr[c];
+                        gw[4 * c] = v.x;
+                        gw[4 * c + 1] = v.y;
+                        gw[4 * c + 2] = v.z;
+                        gw[4 * c + 3] = v.w;
+                    }
                 }
-            }
-            // all 128 threads of the group agree (TMEM loads are warp-collective, the
-            // exchange spans the group)
-            if (!epi_all(a, bar_wait(acc_full(u), uph, limit, s_abort))) { ok = false; break; }
-            tc_fence_after();
-            const unsigned taddr = tmem + ((unsigned)(quarter * 32) << 16) + (unsigned)(u * kBufCols);
-            if (FINAL) {
-                float d0, d1, d2;
-                tmem_ld3(taddr, taddr + NO, taddr + 2 * NO, d0, d1, d2);
-                tc_fence_before();
-                bar_arrive(acc_empty(u));
-                if (lane < 2) {
-                    ex[((quarter * 2 + lane) * 2 + 0) * 32] = d1;
-                    ex[((quarter * 2 + lane) * 2 + 1) * 32] = d2;
-                }
-                epi_sync(a);
-                float s1 = __shfl_down_sync(0xffffffffu, d1, 1);
-                float s2 = __shfl_down_sync(0xffffffffu, d2, 2);
-                if (quarter < 3) {
-                    if (lane == 31) s1 = ex[(((quarter + 1) * 2 + 0) * 2 + 0) * 32];
-                    if (lane >= 30) s2 = ex[(((quarter + 1) * 2 + lane - 30) * 2 + 1) * 32];
-                }
-                if (!zero) {
-                    const long long node = ((long long)i * G.nt + j) * G.np + k;
-                    reinterpret_cast<float *>(out_)[(long long)g * G.nr * G.nt * G.np + node] =
-                        (d0 + s1) + s2 + bz[0];
-                }
-            } else {
-                float d0[32], d1[32], d2[32];
-                {
-                    unsigned r0[32], r1[32], r2[32];
-                    tmem_ld96(taddr, r0, r1, r2);
+                // all 128 threads of the group agree (TMEM loads are warp-collective, the
+                // exchange spans the group)
+                if (!epi_all(a, bar_wait(acc_full(u), uph, limit, s_abort))) { ok = false; break; }
+                tc_fence_after();
+                const unsigned taddr = tmem + ((unsigned)(quarter * 32) << 16) + (unsigned)(u * kBufCols);
+                if (FINAL) {
+                    float d0, d1, d2;
+                    tmem_ld3(taddr, taddr + NO, taddr + 2 * NO, d0, d1, d2);
+                    tc_fence_before();
+                    bar_arrive(acc_empty(u));
+                    if (lane < 2) {
+                        ex[((quarter * 2 + lane) * 2 + 0) * 32] = d1;
+                        ex[((quarter * 2 + lane) * 2 + 1) * 32] = d2;
+                    }
+                    epi_sync(a);
+                    float s1 = __shfl_down_sync(0xffffffffu, d1, 1);
+                    float s2 = __shfl_down_sync(0xffffffffu, d2, 2);
+                    if (quarter < 3) {
+                        if (lane == 31) s1 = ex[(((quarter + 1) * 2 + 0) * 2 + 0) * 32];
+                        if (lane >= 30) s2 = ex[(((quarter + 1) * 2 + lane - 30) * 2 + 1) * 32];
+                    }
+                    if (!zero) {
+                        const long long node = ((long long)i * G.nt + j) * G.np + k;
+                        reinterpret_cast<float *>(out_)[(long long)g * G.nr * G.nt * G.np + node] =
+                            (d0 + s1) + s2 + bz[0];
+                    }
+                } else {
+                    float d0[32], d1[32], d2[32];
+                    {
+                        unsigned r0[32], r1[32], r2[32];
+                        tmem_ld96(taddr, r0, r1, r2);
+#pragma unroll
+                        for (int c = 0; c < 32; ++c) {
+                            d0[c] = __uint_as_float(r0[c]);
+                            d1[c] = __uint_as_float(r1[c]);
+                            d2[c] = __uint_as_float(r2[c]);
+                        }
+                    }
+                    tc_fence_before();
+                    bar_arrive(acc_empty(u));
+                    if (lane < 2) {
+                        float4 *e = reinterpret_cast<float4 *>(ex + (quarter * 2 + lane) * 2 * 32);
+#pragma unroll
+                        for (int c = 0; c < 8; ++c) {
+                            e[c] = make_float4(d1[4 * c], d1[4 * c + 1], d1[4 * c + 2], d1[4 * c + 3]);
+                            e[8 + c] = make_float4(d2[4 * c], d2[4 * c + 1], d2[4 * c + 2], d2[4 * c + 3]);
+                        }
+                    }
+                    epi_sync(a);
 #pragma unroll
                     for (int c = 0; c < 32; ++c) {
-                        d0[c] = __uint_as_float(r0[c]);
-                        d1[c] = __uint_as_float(r1[c]);
-                        d2[c] = __uint_as_float(r2[c]);
+                        d1[c] = __shfl_down_sync(0xffffffffu, d1[c], 1);
+                        d2[c] = __shfl_down_sync(0xffffffffu, d2[c], 2);
                     }
-                }
-                tc_fence_before();
-                bar_arrive(acc_empty(u));
-                if (lane < 2) {
-                    float4 *e = reinterpret_cast<float4 *>(ex + (quarter * 2 + lane) * 2 * 32);
+                    if (lane >= 30 && quarter < 3) {   // the next quarter's first lanes
+                        const float4 *e1 = reinterpret_cast<const float4 *>(ex + (quarter + 1) * 2 * 2 * 32);
+                        const float4 *e2 = e1 + (lane - 30) * 16 + 8;
 #pragma unroll
-                    for (int c = 0; c < 8; ++c) {
-                        e[c] = make_float4(d1[4 * c], d1[4 * c + 1], d1[4 * c + 2], d1[4 * c + 3]);
-                        e[8 + c] = make_float4(d2[4 * c], d2[4 * c + 1], d2[4 * c + 2], d2[4 * c + 3]);
-                    }
-                }
-                epi_sync(a);
-#pragma unroll
-                for (int c = 0; c < 32; ++c) {
-                    d1[c] = __shfl_down_sync(0xffffffffu, d1[c], 1);
-                    d2[c] = __shfl_down_sync(0xffffffffu, d2[c], 2);
-                }
-                if (lane >= 30 && quarter < 3) {   // the next quarter's first lanes
-                    const float4 *e1 = reinterpret_cast<const float4 *>(ex + (quarter + 1) * 2 * 2 * 32);
-                    const float4 *e2 = e1 + (lane - 30) * 16 + 8;
-#pragma unroll
-                    for (int c = 0; c < 8; ++c) {
-                        const float4 x = e2[c];
-                        d2[4 * c] = x.x;
-                        d2[4 * c + 1] = x.y;
-                        d2[4 * c + 2] = x.z;
-                        d2[4 * c + 3] = x.w;
-                        if (lane == 31) {
-                            const float4 y = e1[c];
-                            d1[4 * c] = y.x;
-                            d1[4 * c + 1] = y.y;
-                            d1[4 * c + 2] = y.z;
-                            d1[4 * c + 3] = y.w;
+                        for (int c = 0; c < 8; ++c) {
+                            const float4 x = e2[c];
+                            d2[4 * c] = x.x;
+                            d2[4 * c + 1] = x.y;
+                            d2[4 * c + 2] = x.z;
+                            d2[4 * c + 3] = x.w;
+                            if (lane == 31) {
+                                const float4 y = e1[c];
+                                d1[4 * c] = y.x;
+                                d1[4 * c + 1] = y.y;
+                                d1[4 * c + 2] = y.z;
+                                d1[4 * c + 3] = y.w;
+                            }
                         }
                     }
-                }
-                unsigned w[16];
+                    unsigned w[16];
 #pragma unroll
-                for (int c = 0; c < 32; c += 2) {
-                    float v[2];
+                    for (int c = 0; c < 32; c += 2) {
+                        float v[2];
 #pragma unroll
-                    for (int h = 0; h < 2; ++h) {
-                        const float sum = (d0[c + h] + d1[c + h]) + d2[c + h];
-                        if (MODE == kEpiGate) {
-                            const unsigned short hb = (unsigned short)(gw[c / 2] >> (16 * h));
-                            const bool open = !zero && __bfloat162float(__ushort_as_bfloat16(hb)) > 0.0f;
-                            v[h] = open ? sum : 0.0f;
-                        } else {
-                            v[h] = zero ? 0.0f : fmaxf(sum + bz[c + h], 0.0f);
+                        for (int h = 0; h < 2; ++h) {
+                            const float sum = (d0[c + h] + d1[c + h]) + d2[c + h];
+                            if (MODE == kEpiGate) {
+                                const unsigned short hb = (unsigned short)(gw[c / 2] >> (16 * h));
+                                const bool open = !zero && __bfloat162float(__ushort_as_bfloat16(hb)) > 0.0f;
+                                v[h] = open ? sum : 0.0f;
+                            } else {
+                                v[h] = zero ? 0.0f : fmaxf(sum + bz[c + h], 0.0f);
+                            }
                         }
+                        const __nv_bfloat162 p = __floats2bfloat162_rn(v[0], v[1]);
+                        w[c / 2] = *reinterpret_cast<const unsigned *>(&p);
                     }
-                    const __nv_bfloat162 p = __floats2bfloat162_rn(v[0], v[1]);
-                    w[c / 2] = *reinterpret_cast<const unsigned *>(&p);
-                }
-                if (out_ok) {
-                    uint4 *o = reinterpret_cast<uint4 *>(out_) + ((long long)g * G.R + n) * 4;
+                    if (out_ok) {
+                        uint4 *o = reinterpret_cast<uint4 *>(out_) + ((long long)g * G.R + n) * 4;
 #pragma unroll
-                    for (int c = 0; c < 4; ++c)
-                        o[c] = make_uint4(w[4 * c], w[4 * c + 1], w[4 * c + 2], w[4 * c + 3]);
+                        for (int c = 0; c < 4; ++c)
+                            o[c] = make_uint4(w[4 * c], w[4 * c + 1], w[4 * c + 2], w[4 * c + 3]);
+                    }
                 }
             }
-          }
         }
     }
     tc_fence_before();

@@ -63,3 +63,40 @@ def test_training_gradient_matches_the_fp32_path(shape, n):
     ctx.close()
     assert abs(loss / want - 1) <= 16 * 2.0 ** -9
     assert ((g - ref).abs() <= 16 * 2.0 ** -9 * ref).all()
+
+
+@pytest.mark.parametrize("shape,n", [((4, 5, 4), 1), ((5, 4, 66), 33), ((6, 7, 68), 40), ((9, 8, 131), 3)])
+def test_coarse_prediction_is_interpolated(shape, n):
+    """The warm start from every other node (33 and 65 cells along phi, 33 and more sources, odd and even
+    extents) against the network's own prediction, clamped and interpolated in 64 bits: eight products and
+    sums of values up to 1 in FP32, and 1 + v."""
+    import torch
+    import paper_2412_00031_gb300 as tt
+    ctx, theta, _, _ = _setup(tt, shape, n)
+    rng = np.random.default_rng(n)
+    src = rng.uniform(0.1, 0.9, (n, 3)) * np.array([10.0, 0.5, 0.5])
+    model = [torch.full(shape, v, device="cuda") for v in (0.2, 0.01, -0.01)]
+    tt.tt_net_set_stride(ctx, 2)
+    tt.tt_net_set_weights(ctx, theta)
+    net = tuple(s // 2 + 1 for s in shape)
+    x = torch.empty((n, int(np.prod(net)), tt.NET_FEATURES), device="cuda")
+    tt.tt_net_features(ctx, model, src, x)
+    y = torch.empty((n, int(np.prod(net))), device="cuda")
+    tt.tt_net_infer(ctx, x, y)
+    tau = torch.empty(shape + (n,), device="cuda")
+    tt.tt_net_start(ctx, model, src, tau)
+    ctx.close()
+    v = y.double().cpu().numpy().reshape((n,) + net).clip(-0.5, 1.0)
+    for axis, s in enumerate(shape):
+        at = np.minimum(2 * np.arange(net[axis]), s - 1)
+        a = np.minimum(np.arange(s) // 2, net[axis] - 2)
+        f = (np.arange(s) - at[a]) / (at[a + 1] - at[a])
+        f = f.reshape([-1 if k == axis + 1 else 1 for k in range(4)])
+        v = (1 - f) * v.take(a, axis + 1) + f * v.take(a + 1, axis + 1)
+    # the nodes around a source are fixed at 1
+    pos = np.stack([(10.0 - src[:, 0]) / 10.0, src[:, 1] / 0.5, src[:, 2] / 0.5], 1) * (np.array(shape) - 1)
+    near = np.floor(pos + 0.5).astype(int)
+    err = np.abs(tau.cpu().numpy() - 1 - np.moveaxis(v, 0, 3))
+    for b in range(n):
+        err[tuple(slice(max(c - 1, 0), c + 2) for c in near[b]) + (b,)] = 0
+    assert err.max() <= 24 * 2.0 ** -24

@@ -213,16 +213,30 @@ __global__ void __launch_bounds__(kMseThreads)
     }
 }
 
-// Stage 2 (one thread, fixed order): loss and 1 / sum(mask) into scratch[2 * kMseBlocks].
-__global__ void mse_final_kernel(double *__restrict__ scratch, double *__restrict__ loss) {
+// Stage 2 (one block, fixed order): loss and 1 / sum(mask) into scratch[2 * kMseBlocks]. (A single
+// thread's 2,048 dependent FP64 loads and adds took 104 us of a training step.)
+__global__ void __launch_bounds__(kMseThreads) mse_final_kernel(double *__restrict__ scratch, double *__restrict__ loss) {
+    __shared__ double s_a[kMseThreads], s_c[kMseThreads];
     double a = 0.0, c = 0.0;
-    for (int q = 0; q < kMseBlocks; ++q) {
+    for (int q = threadIdx.x; q < kMseBlocks; q += kMseThreads) {
         a += scratch[q];
         c += scratch[kMseBlocks + q];
     }
-    const double inv = a > 0.0 ? 1.0 / a : 0.0;
-    *loss = c * inv;
-    scratch[2 * kMseBlocks] = inv;
+    s_a[threadIdx.x] = a;
+    s_c[threadIdx.x] = c;
+    __syncthreads();
+    for (int h = kMseThreads / 2; h > 0; h >>= 1) {
+        if (threadIdx.x < h) {
+            s_a[threadIdx.x] += s_a[threadIdx.x + h];
+            s_c[threadIdx.x] += s_c[threadIdx.x + h];
+        }
+        __syncthreads();
+    }
+    if (threadIdx.x == 0) {
+        const double inv = s_a[0] > 0.0 ? 1.0 / s_a[0] : 0.0;
+        *loss = s_c[0] * inv;
+        scratch[2 * kMseBlocks] = inv;
+    }
 }
 
 __global__ void mse_grad_kernel(long long total, const float *__restrict__ y,
@@ -409,7 +423,7 @@ cudaError_t run_conv3d_flip(int cin, int cout, const float *w, float *wt, cudaSt
 cudaError_t run_mse(long long total, const float *y, const float *target, const float *mask,
                     float *dy, double *scratch, double *loss, cudaStream_t st) {
     mse_partial_kernel<<<kMseBlocks, kMseThreads, 0, st>>>(total, y, target, mask, scratch);
-    mse_final_kernel<<<1, 1, 0, st>>>(scratch, loss);
+    mse_final_kernel<<<1, kMseThreads, 0, st>>>(scratch, loss);
     mse_grad_kernel<<<blocks_of(total, 256), 256, 0, st>>>(total, y, target, mask, scratch, dy);
     return cudaGetLastError();
 }

@@ -239,7 +239,7 @@ def run_e2e(gp, w, steps):
 
 def kernel_source_digest():
     h = hashlib.sha256()
-    for name in ("tt_sweep.cu", "tt_common.cuh", "tt_internal.h"):
+    for name in ("tt_plane.cu", "tt_plane.cuh", "tt_update.cuh", "tt_common.cuh", "tt_internal.h"):
         with open(os.path.join(ROOT, "paper_2412_00031_gb300", "csrc", name), "rb") as f:
             h.update(f.read())
     return h.hexdigest()[:16]
@@ -347,7 +347,7 @@ def gpu_arm(args, rank, world):
         "config": workload_config(w, world),
         "step_form": ("one captured CUDA graph per step (tt_plan)" if args.plan
                       else "four C-ABI calls per step"),
-        "roofline": {"bound": "hbm", "kernel": "fwd_sweep_kernel<float>", "achieved": f_gbs,
+        "roofline": {"bound": "hbm", "kernel": "plane_kernel<float, 0, 2>", "achieved": f_gbs,
                      "peak": hbm, "peak_kind": peak_kind, "unit": "GB/s", "frac": f_gbs / hbm,
                      "traffic": traffic, "algorithmic_bytes_per_launch": f_bytes,
                      "launch_ms": f_ms, "kernel_source_digest": digest},
@@ -460,7 +460,7 @@ def godunov_leg(args, gp, world):
     fwd_kernel = hbm_kernel(f_ms, float(np.mean([s["node_updates"] for s in fwd])),
                             float(np.mean([s["node_sweeps"] for s in fwd])),
                             FWD_BYTES_PER_UPDATE, FWD_BYTES_PER_NODE_SWEEP, hbm)
-    fwd_kernel["kernel"] = "fwd_sweep_kernel<float, unsigned, 0, 2>"
+    fwd_kernel["kernel"] = "plane_kernel<float, 2, 2>"
     # The same forward from tau = 1 (opts.init = 0), for comparison with the start from above.
     o1 = tt.default_opts(tt.TT_F32, scheme=2, fwd_groups=gp.opts.fwd_groups)
     it1 = tt.tt_forward(gp.ctx, gp.model, gp.w.src, gp.tau, None, o1)

@@ -188,10 +188,9 @@ __global__ void __launch_bounds__(kPlaneThreads, 1)
         F v[7][NS];
         typename U::Fac fc;
         NodeRec<F> rec;
-        Node d;
         F *p = nullptr;
         auto load = [&]() {
-            d = place(o, pk);
+            const Node d = place(o, pk);
             p = a.tau + (d.n * B + b);
             ld_pack(p, v[0]);
             ld_pack(p + osr, v[1]);
@@ -215,8 +214,10 @@ __global__ void __launch_bounds__(kPlaneThreads, 1)
             if (any && slot < np.total()) pkn = sch.entry(np, slot, on);
             if (mine)
                 for (int x = slot;;) {
-                    const bool rr = o & 4, rt = o & 2, rp = o & 1;
-                    const bool face = pk & 0x40000000u;
+                    const int ox = o;
+                    // A face finds the node's place again: its indices held over the update cost spills
+                    // (Godunov pairs 182 -> 134 B; 121x161x161 x 256 sources, whole step 755 -> 740 ms).
+                    const unsigned pkx = pk;
                     x += slots;
                     if (x < total) pk = sch.entry(cp, x, o);
                     F tn[NS];
@@ -228,7 +229,9 @@ __global__ void __launch_bounds__(kPlaneThreads, 1)
                     if (moved) st_pack(p, tn);
                     // a layer next to a face (second in the ordering: the entry face, last: the
                     // exit face) along some axis
-                    if (SCHEME != 3 && face) {
+                    if (SCHEME != 3 && (pkx & 0x40000000u)) {
+                        const Node d = place(ox, pkx);
+                        const bool rr = ox & 4, rt = ox & 2, rp = ox & 1;
 #pragma unroll
                         for (int h = 0; h < NS; ++h) {
                             if (!act[h]) continue;

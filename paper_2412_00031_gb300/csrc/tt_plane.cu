@@ -166,7 +166,7 @@ __global__ void __launch_bounds__(kPlaneThreads, 1)
         // most), concatenated; this thread takes the nodes slot, slot + slots, ... The list is
         // static: the next entry is looked up while a node is updated, the next time step's first
         // one before the barrier.
-        Planes cp, np;
+        Planes cp;
         auto place = [&](int o, unsigned pk) {
             Node d;
             d.aa = (int)(pk >> 20) & 1023;
@@ -208,10 +208,13 @@ __global__ void __launch_bounds__(kPlaneThreads, 1)
             if (mine) load();
             // the next time step's planes and this thread's first node there: static, and looked
             // up while the loads above are on their way
-            sch.planes(np, tau + 1, cp.o0);
             int on = 0;
             unsigned pkn = 0;
-            if (any && slot < np.total()) pkn = sch.entry(np, slot, on);
+            {
+                Planes np;
+                sch.planes(np, tau + 1, cp.o0);
+                if (any && slot < np.total()) pkn = sch.entry(np, slot, on);
+            }
             if (mine)
                 for (int x = slot;;) {
                     const int ox = o;
@@ -253,10 +256,12 @@ __global__ void __launch_bounds__(kPlaneThreads, 1)
                     if (x >= total) break;
                     load();
                 }
+            // again: held over the updates they cost spills (LF pairs 100 -> 12 B; 121x161x161 x 256
+            // sources 2793 -> 2644 ms, Godunov 436 -> 423)
+            sch.planes(cp, tau + 1, cp.o0);
             if (!grid_barrier(bar, a.spin_ns, nblk)) return;
             o = on;
             pk = pkn;
-            cp = np;
         }
         // 1: the source has not converged (three words a source, by iteration)
         int *flag = m.moved + (it % 3) * a.src_n;

@@ -360,11 +360,16 @@ template <typename F> __global__ void edge_kernel(FwdArgs<F> a, int axis) {
     *p = fmax_((F)2 * t1 - t2, t2);
 }
 
+// Threads of the adjoint: FP32 fits 64 registers without spills, and 32 warps an SM hide more of its
+// 14 loads an update than 24: 121x161x161 x 256 sources 319 -> 284 ms. (The forward kernels spill at
+// 64: 2644 -> 2694 ms, Godunov 423 -> 445.)
+template <typename F> constexpr int kAdjThreads = sizeof(F) == 4 ? 1024 : kPlaneThreads;
+
 // The adjoint sweep (Eq. 5) from the face coefficients (adj_coef_kernel, face_update), over every
 // node, in the same organisation; no faces to complete. emax: [3][2][src_n], by iteration mod 3 the
 // sources' largest |change| of P and, in the last ordering, largest |P|.
 template <typename F, int NS>
-__global__ void __launch_bounds__(kPlaneThreads, 1) adj_plane_kernel(AdjArgs<F> a, PlaneShape m, F *emax) {
+__global__ void __launch_bounds__(kAdjThreads<F>, 1) adj_plane_kernel(AdjArgs<F> a, PlaneShape m, F *emax) {
     extern __shared__ __align__(8) int s_off[];
     __shared__ int s_units, s_start[8];
     const GridC &g = a.g;
@@ -536,7 +541,7 @@ cudaError_t run_plane_forward(FwdArgs<F> a, int groups, int *moved, int n_sm, in
     if constexpr (sizeof(F) == 4)
         if (pair) fn = plane_ptr<F, 2>(a.scheme);
     const size_t smem = sizeof(int) * (a.n_planes + 1 + 2 * (size_t)n) + n;
-    if ((e = plane_shape(m, fn, smem, a.na, a.nb, a.nc, n, pair ? 2 : 1, groups, n_sm, launch_blocks, grid, block)) != cudaSuccess)
+    if ((e = plane_shape(m, fn, smem, a.na, a.nb, a.nc, n, pair ? 2 : 1, groups, kPlaneThreads, n_sm, launch_blocks, grid, block)) != cudaSuccess)
         return e;
     *kernels = tele ? 1 : 4;
     m.moved = moved;
@@ -573,7 +578,7 @@ cudaError_t run_plane_adjoint(AdjArgs<F> a, int groups, F *emax, int n_sm, int l
     if constexpr (sizeof(F) == 4)
         if (pair) fn = (const void *)adj_plane_kernel<F, 2>;
     const size_t smem = sizeof(int) * (a.n_planes + 2 + (size_t)n) + 2 * sizeof(F) * (size_t)n + n;
-    if ((e = plane_shape(m, fn, smem, a.g.nr, a.g.nt, a.g.np, n, pair ? 2 : 1, groups, n_sm, launch_blocks, grid, block)) != cudaSuccess)
+    if ((e = plane_shape(m, fn, smem, a.g.nr, a.g.nt, a.g.np, n, pair ? 2 : 1, groups, kAdjThreads<F>, n_sm, launch_blocks, grid, block)) != cudaSuccess)
         return e;
     if ((e = cudaMemsetAsync(emax, 0, sizeof(F) * 6 * (size_t)n, st)) != cudaSuccess) return e;
     void *args[] = {&a, &m, &emax};

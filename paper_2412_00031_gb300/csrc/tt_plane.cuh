@@ -107,14 +107,14 @@ inline bool plane_pairs(const PlaneShape &m, int na, int nb, int nc, int n, int 
 // barrier of 608 blocks takes 2.5 us, of 152 1.6 us); no more threads than the widest plane has
 // nodes and sources. cudaErrorInvalidConfiguration: the sources exceed one resident launch.
 inline cudaError_t plane_shape(PlaneShape &m, const void *fn, size_t smem, int na, int nb, int nc, int n, int ns,
-                               int groups, int n_sm, int launch_blocks, int *grid, int *block) {
+                               int groups, int max_threads, int n_sm, int launch_blocks, int *grid, int *block) {
     cudaError_t e;
     if ((e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess)
         return e;
     if (groups <= 0) groups = 1;
     if (groups > kMaxBarrierGroups) groups = kMaxBarrierGroups;
     if (groups > (n + 31) / 32) groups = (n + 31) / 32;
-    int threads = kPlaneThreads / groups / 32 * 32;
+    int threads = max_threads / groups / 32 * 32;
     const int ext[3] = {na, nb, nc};
     long long widest = 0;
     for (int x = 0; x < 3; ++x)

@@ -211,11 +211,9 @@ __global__ void __launch_bounds__(kPlaneThreads, 1)
             // up while the loads above are on their way
             int on = 0;
             unsigned pkn = 0;
-            {
-                Planes np;
-                sch.planes(np, tau + 1, cp.o0);
-                if (any && slot < np.total()) pkn = sch.entry(np, slot, on);
-            }
+            Planes np;
+            sch.planes(np, tau + 1, cp.o0);
+            if (any && slot < np.total()) pkn = sch.entry(np, slot, on);
             if (mine)
                 for (int x = slot;;) {
                     const int ox = o;
@@ -259,7 +257,9 @@ __global__ void __launch_bounds__(kPlaneThreads, 1)
                 }
             // again: held over the updates they cost spills (LF pairs 100 -> 12 B; 121x161x161 x 256
             // sources 2793 -> 2644 ms, Godunov 436 -> 423)
-            sch.planes(cp, tau + 1, cp.o0);
+            // One FP32 source a thread has the registers, and its short steps no time for the lookup.
+            if constexpr (NS == 1 && sizeof(F) == 4) cp = np;
+            else sch.planes(cp, tau + 1, cp.o0);
             if (!grid_barrier(bar, a.spin_ns, nblk)) return;
             o = on;
             pk = pkn;

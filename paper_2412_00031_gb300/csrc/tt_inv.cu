@@ -98,8 +98,9 @@ __global__ void normalize_kernel(long long N, double *Ks, double *Kxi, double *K
 // dV = h2(i)^2 cos(theta_j) dr dtheta dphi. A warp takes a row, a lane the outputs (h, c) of
 // which it sums only the nodes under the hat, [rng[2 (h, c)], rng[2 (h, c) + 1]): the other
 // weights are zero (a dense sum over the row, 9 / 2 times the FP64 work, took 0.4 ms per kernel
-// at 101x201x201 and 5 grids of 11^3). In the dense sum a value that is not finite reaches
-// every output of its row (times a zero weight); `rest` adds that.
+// at 101x201x201 and 5 grids of 11^3). A row with a value that is not finite takes the dense sum:
+// there the value reaches every output, infinite under its hats and NaN (times a zero weight)
+// elsewhere. `rest`, the sum of 0 times the values, is NaN for such a row and 0 for the others.
 constexpr int kProjRows = 4;   // rows (warps) of a block
 __global__ void __launch_bounds__(32 * kProjRows)
     project_phi_kernel(MgDims d, const double *__restrict__ K, const double *__restrict__ h2,
@@ -122,9 +123,9 @@ __global__ void __launch_bounds__(32 * kProjRows)
     const double dV = h2[i] * h2[i] * cost[j] * dvol;
     for (int q = lane; q < d.H * d.cp; q += 32) {
         const double *wt = Wp + (long long)q * d.np;
-        const int k1 = rng[2 * q + 1];
-        double acc = rest;
-        for (int k = rng[2 * q]; k < k1; ++k) acc += row[k] * wt[k];
+        const int k0 = rest == 0.0 ? rng[2 * q] : 0, k1 = rest == 0.0 ? rng[2 * q + 1] : d.np;
+        double acc = 0.0;
+        for (int k = k0; k < k1; ++k) acc += row[k] * wt[k];
         const int h = q / d.cp, c = q - h * d.cp;
         T1[(((long long)h * d.nr + i) * d.nt + j) * d.cp + c] = acc * dV;
     }

@@ -101,6 +101,10 @@ constexpr int kFlagInts = 6;
 constexpr size_t kCoefBudgetBytes = 64ull << 30;
 // Largest factor cache (1/T0 and grad T0 / T0 per node and source) one forward slice keeps.
 constexpr size_t kFactorCacheBudgetBytes = 32ull << 30;
+// Node constants of a 2-D teleseismic launch: the most that one takes (further events follow in
+// launches of their own), and the most that the context keeps; what is larger is given back when
+// the call returns, so that it takes no memory from later calls' workspaces.
+constexpr size_t kTelePreBudgetBytes = 32ull << 30, kTelePreKeepBytes = 1ull << 30;
 tt_status fail(tt_ctx *c, tt_status s, const char *fmt, ...) {
     if (c) {
         va_list ap;
@@ -119,19 +123,30 @@ tt_status fail(tt_ctx *c, tt_status s, const char *fmt, ...) {
                         cudaGetErrorString(e_));                                      \
     } while (0)
 
-tt_status ensure(tt_ctx *ctx, DevBuf &b, size_t bytes) {
-    if (bytes <= b.bytes) return TT_OK;
+bool grow(DevBuf &b, size_t bytes) {
+    if (bytes <= b.bytes) return true;
     if (b.p) cudaFree(b.p);
     b.p = nullptr;
     b.bytes = 0;
-    size_t want = bytes < 256 ? 256 : bytes;
-    if (cudaMalloc(&b.p, want) != cudaSuccess) {
+    if (cudaMalloc(&b.p, bytes) != cudaSuccess) {
         cudaGetLastError();
-        return fail(ctx, TT_ENOMEM, "workspace allocation of %zu bytes failed", want);
+        return false;
     }
-    b.bytes = want;
-    return TT_OK;
+    b.bytes = bytes;
+    return true;
 }
+
+tt_status ensure(tt_ctx *ctx, DevBuf &b, size_t bytes) {
+    const size_t want = bytes < 256 ? 256 : bytes;
+    return grow(b, want) ? TT_OK : fail(ctx, TT_ENOMEM, "workspace allocation of %zu bytes failed", want);
+}
+
+// A buffer of one call.
+struct CallBuf : DevBuf {
+    ~CallBuf() {
+        if (p) cudaFree(p);
+    }
+};
 
 #define ENSURE(buf, bytes)                        \
     do {                                          \
@@ -1539,14 +1554,27 @@ tt_status tt_tele2d(tt_ctx *ctx, int dtype, int n_r, int n_d, double r_min_km, d
     CK(cudaMemcpyAsync(d_rs, h_r_src_km, sizeof(double) * n_ev, cudaMemcpyHostToDevice, ctx->st));
     const double dr = (r_max_km - r_min_km) / (n_r - 1);
     const double dd = d_max_deg * (3.14159265358979323846 / 180.0) / (n_d - 1);
-    // the nodes' constants, where they fit: the solve runs without them too
-    void *pre = ensure(ctx, ctx->tele_pre, 4 * fs * (size_t)n_ev * n_r * n_d) == TT_OK ? ctx->tele_pre.p
-                                                                                       : nullptr;
-    CK(dtype == TT_F32 ? run_tele2d<float>(n_r, n_d, r_min_km, dr, dd, d_s_r, d_rs, n_ev, tol,
-                                           max_iter, ctx->tele_tau.p, pre, d_T, d_it, ctx->n_sm, ctx->st)
-                       : run_tele2d<double>(n_r, n_d, r_min_km, dr, dd, d_s_r, d_rs, n_ev, tol,
-                                            max_iter, ctx->tele_tau.p, pre, d_T, d_it, ctx->n_sm, ctx->st));
-    ctx->launches += 1;
+    // The nodes' constants of a slice of the events, where they fit: the solve runs without them
+    // too, then all events together. (So also where the slices would leave most SMs idle: the
+    // constants halve an update, and an event has at most 8 blocks.)
+    const size_t nn = (size_t)n_r * n_d;
+    int slice = 4 * fs * nn * n_ev > kTelePreBudgetBytes ? (int)(kTelePreBudgetBytes / (4 * fs * nn)) : n_ev;
+    CallBuf own;
+    void *pre = nullptr;
+    if (slice == n_ev || 8LL * slice >= ctx->n_sm) {
+        DevBuf &b = 4 * fs * nn * slice > kTelePreKeepBytes ? own : ctx->tele_pre;
+        if (grow(b, 4 * fs * nn * slice)) pre = b.p;
+    }
+    if (!pre) slice = n_ev;
+    for (int e = 0; e < n_ev; e += slice) {
+        const int n = slice < n_ev - e ? slice : n_ev - e;
+        void *tau = (char *)ctx->tele_tau.p + fs * nn * e, *T = (char *)d_T + fs * nn * e;
+        CK(dtype == TT_F32 ? run_tele2d<float>(n_r, n_d, r_min_km, dr, dd, d_s_r, d_rs + e, n, tol, max_iter,
+                                               tau, pre, T, d_it + e, ctx->n_sm, ctx->st)
+                           : run_tele2d<double>(n_r, n_d, r_min_km, dr, dd, d_s_r, d_rs + e, n, tol, max_iter,
+                                                tau, pre, T, d_it + e, ctx->n_sm, ctx->st));
+        ctx->launches += 1;
+    }
     std::vector<int> it(n_ev);
     CK(cudaMemcpyAsync(it.data(), d_it, sizeof(int) * n_ev, cudaMemcpyDeviceToHost, ctx->st));
     CK(cudaStreamSynchronize(ctx->st));

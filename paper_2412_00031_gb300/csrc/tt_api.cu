@@ -1561,7 +1561,7 @@ tt_status tt_tele2d(tt_ctx *ctx, int dtype, int n_r, int n_d, double r_min_km, d
     int slice = 4 * fs * nn * n_ev > kTelePreBudgetBytes ? (int)(kTelePreBudgetBytes / (4 * fs * nn)) : n_ev;
     CallBuf own;
     void *pre = nullptr;
-    if (slice == n_ev || 8LL * slice >= ctx->n_sm) {
+    if (tele2d_pre(dtype == TT_F64, n_r, n_d) && (slice == n_ev || 8LL * slice >= ctx->n_sm)) {
         DevBuf &b = 4 * fs * nn * slice > kTelePreKeepBytes ? own : ctx->tele_pre;
         if (grow(b, 4 * fs * nn * slice)) pre = b.p;
     }

@@ -22,7 +22,7 @@ namespace ttgb {
 
 namespace {
 
-constexpr int kTeleThreads = 512;   // of an event, over the blocks of its cluster
+constexpr int kTeleThreads = 512;   // of an event, over up to four blocks (1024 over eight)
 constexpr int kTeleCluster = 8;
 
 template <typename F>
@@ -115,13 +115,14 @@ __device__ F god2d(const Vec4<F> &q, F e0, F tc, F lo0, F hi0, F lo1, F hi1) {
     return found ? add_(tc, div_(bestN, bestD)) : tc;
 }
 
-// PRE: the constants of every node are computed once and kept in `pre` [n_ev][n_r][n_d]; in FP64
-// they are three quarters of an update's instructions on a pipe of 2 lanes a clock and SM, and an
-// iteration updates a node four times (24 events of 201 x 401 nodes with the region's 81x101x101
-// solve: 1129 -> 674 ms, with the clusters below). Without it (no memory for `pre`) every update computes
-// them; the bits are the same.
+// PRE: the constants of every node are computed once and kept in `pre` [n_ev][n_r][n_d]; without
+// it every update computes them; the bits are the same. In FP64 they are three quarters of an
+// update's instructions on a pipe of 2 lanes a clock and SM, and an iteration updates a node four
+// times (24 events of 201x401 nodes, 12 iterations: 246 -> 110 ms with the clusters below).
 // CL: blocks of an event. A diagonal of a few hundred nodes keeps one SM's FP64 pipe busy for a few
 // microseconds; spread over a cluster it costs little more than the barrier.
+// In FP32 the constants cost less than reading them back and the barrier is the longer part of a
+// step: tele2d_pre and tele2d_blocks.
 template <typename F, bool PRE, int CL>
 __global__ void __launch_bounds__(kTeleThreads / (CL > 4 ? 4 : CL))
 tele2d_kernel(int n_r, int n_d, F r_min, F dr, F dd, const F *s_r, const double *r_src,
@@ -166,10 +167,11 @@ tele2d_kernel(int n_r, int n_d, F r_min, F dr, F dd, const F *s_r, const double 
                     const int j = up_j ? b : n_d - 2 - b;
                     if (abs(i - is) <= 1 && j <= 1) continue;
                     const long long c = (long long)i * n_d + j;
-                    const F tc = tau[c];
+                    // the loads first: the constants' arithmetic runs while they are on their way
+                    const F tc = tau[c], lo0 = tau[c - n_d], hi0 = tau[c + n_d];
+                    const F lo1 = tau[(long long)i * n_d + (j > 0 ? j - 1 : 1)], hi1 = tau[c + 1];
                     const Vec4<F> k = PRE ? pre[c] : node_consts<F>(n_r, r_min, dr, dd, s_r, r_s, s_s, i, j);
-                    const F v = god2d<F>(k, e0, tc, tau[c - n_d], tau[c + n_d],
-                                         tau[(long long)i * n_d + (j > 0 ? j - 1 : 1)], tau[c + 1]);
+                    const F v = god2d<F>(k, e0, tc, lo0, hi0, lo1, hi1);
                     err = fmax(err, fabs(v - tc));
                     tau[c] = v;
                 }
@@ -298,6 +300,20 @@ static cudaError_t launch_tele2d_cl(int n_r, int n_d, double r_min, double dr, d
                               r_src, (F)tol, max_iter, (F *)tau, (Vec4<F> *)pre, (F *)T, iters);
 }
 
+// The constants are kept in FP64, and in FP32 only where an event's stay in an SM's L1. FP32, ms of
+// 6 iterations without / with them: 21x31 x 100 events 0.70 / 0.46; 201x401 x 10 10.3 / 10.3, x 152
+// 10.3 / 12.4; 1001x2001 x 10 124 / 156.
+bool tele2d_pre(bool f64, int n_r, int n_d) { return f64 || 16LL * n_r * n_d <= 128 << 10; }
+
+// Blocks of an event: as many as the SMs have room for in FP64. In FP32 eight where a diagonal has
+// 768 nodes or more (one block takes it in two rounds), otherwise one. FP32, ms of 6 iterations, one
+// / eight blocks: 201x401 x 10 events 10.3 / 18.5; 601x1201 x 10 54.7 / 63.9; 801x1601 x 10 102 / 89;
+// 1001x2001 x 19 127 / 132; 2001x2001 x 19 261 / 222; 4001x4001 x 1 1134 / 554.
+static int tele2d_blocks(bool f64, int n_r, int n_d, int n_ev, int n_sm) {
+    if (!f64) return 8 * n_ev <= n_sm && n_r - 2 >= 768 && n_d - 1 >= 768 ? 8 : 1;
+    return 8 * n_ev <= n_sm ? 8 : 4 * n_ev <= n_sm ? 4 : 2 * n_ev <= n_sm ? 2 : 1;
+}
+
 template <typename F, bool PRE>
 static cudaError_t launch_tele2d(int cl, int n_r, int n_d, double r_min, double dr, double dd, const void *s_r,
                                  const double *r_src, int n_ev, double tol, int max_iter, void *tau,
@@ -305,9 +321,13 @@ static cudaError_t launch_tele2d(int cl, int n_r, int n_d, double r_min, double 
 #define TTGB_TELE_CL(CL)                                                                               \
     return launch_tele2d_cl<F, PRE, CL>(n_r, n_d, r_min, dr, dd, s_r, r_src, n_ev, tol, max_iter, tau, \
                                         pre, T, iters, st)
-    if (cl == 8) TTGB_TELE_CL(8);
-    if (cl == 4) TTGB_TELE_CL(4);
-    if (cl == 2) TTGB_TELE_CL(2);
+    constexpr bool kF64 = sizeof(F) == 8;
+    if constexpr (kF64 || !PRE)
+        if (cl == 8) TTGB_TELE_CL(8);
+    if constexpr (kF64) {
+        if (cl == 4) TTGB_TELE_CL(4);
+        if (cl == 2) TTGB_TELE_CL(2);
+    }
     TTGB_TELE_CL(1);
 #undef TTGB_TELE_CL
 }
@@ -316,8 +336,7 @@ template <typename F>
 cudaError_t run_tele2d(int n_r, int n_d, double r_min, double dr, double dd, const void *s_r,
                        const double *r_src, int n_ev, double tol, int max_iter, void *tau,
                        void *pre, void *T, int *iters, int n_sm, cudaStream_t st) {
-    // as many blocks an event as the SMs have room for
-    const int cl = 8 * n_ev <= n_sm ? 8 : 4 * n_ev <= n_sm ? 4 : 2 * n_ev <= n_sm ? 2 : 1;
+    const int cl = tele2d_blocks(sizeof(F) == 8, n_r, n_d, n_ev, n_sm);
     cudaError_t e = pre ? launch_tele2d<F, true>(cl, n_r, n_d, r_min, dr, dd, s_r, r_src, n_ev, tol, max_iter, tau, pre, T, iters, st)
                         : launch_tele2d<F, false>(cl, n_r, n_d, r_min, dr, dd, s_r, r_src, n_ev, tol, max_iter, tau, pre, T, iters, st);
     if (e != cudaSuccess) return e;

@@ -7,6 +7,8 @@
 
 namespace ttgb {
 
+// The 2-D solve of this type and grid takes the nodes' constants (run_tele2d's pre).
+bool tele2d_pre(bool f64, int n_r, int n_d);
 // 2-D traveltimes of n_ev events (a block or a cluster of blocks each) on r = r_min + i dr,
 // Delta = j dd: s_r [n_r] of F, r_src [n_ev] double, tau scratch and T [n_ev][n_r][n_d] of F,
 // iters [n_ev]; pre: scratch of four F per node and event for the nodes' constants, or NULL

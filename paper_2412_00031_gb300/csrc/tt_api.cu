@@ -940,10 +940,10 @@ tt_status enq_kernel(tt_ctx *ctx, const tt_model *m, int B, const void *d_T, con
     ctx->kacc_B = B;
     if (m->dtype == TT_F32)
         CK(run_kernel_accum<float>(ctx->g, B, m->d_s, d_T, d_P, ctx->gd.h2, ctx->gd.cost, Ks, Kxi,
-                                   Keta, ctx->st));
+                                   Keta, ctx->n_sm, ctx->st));
     else
         CK(run_kernel_accum<double>(ctx->g, B, m->d_s, d_T, d_P, ctx->gd.h2, ctx->gd.cost, Ks,
-                                    Kxi, Keta, ctx->st));
+                                    Kxi, Keta, ctx->n_sm, ctx->st));
     CK(record(ctx, ctx->ev_kacc[1]));
     ctx->launches += 1;
     return TT_OK;

@@ -4,6 +4,8 @@
 // (Eqs. 6-8).
 #include <cuda_runtime.h>
 
+#include <algorithm>
+
 #include "tt_aux.h"
 
 namespace ttgb {
@@ -485,27 +487,28 @@ template <typename F, int VEC> __device__ __forceinline__ void ld_vec(const F *p
     }
 }
 
-// Kernels of Eqs. 6-8. A warp takes 32 consecutive phi nodes of one (r, theta) row, 32 / W of
-// them at a time: W lanes (a power of two) stride over a node's sources, VEC at a time. A lane
+// Kernels of Eqs. 6-8. A warp takes up to 32 consecutive phi nodes of one (r, theta) row (M: a row in
+// equal parts), 32 / W of them at a time: W lanes (a power of two) stride over a node's sources, VEC
+// at a time. A lane
 // forms each source's term in the fields' precision F (reciprocals instead of divisions) and
 // sums its terms with a compensated accumulator in F (TwoSum); the W lanes' accumulators merge
 // in a fixed butterfly. The totals of the 32 nodes are then added to the FP64 kernels by one
 // lane per node.
 //
 // The FP64 pipe (2 lanes a clock and SM) decides the layout: the two reciprocals of the row and
-// the final sums are issued once per 32 nodes, not once per node: 5.31 ms with a warp per node at
-// 121x161x161 nodes x 256 sources, 1.97 ms now (the fields' 6.4 GB once: 0.95 ms).
+// the final sums are issued once per M nodes, not once per node: 5.31 ms with a warp per node at
+// 121x161x161 nodes x 256 sources, 1.84 ms now (the fields' 6.4 GB once: 0.95 ms).
 // Fewer than 32 sources leave no lane idle: W shrinks and a warp takes several nodes at once.
 template <typename F, int VEC>
 __global__ void __launch_bounds__(256)
-    kernel_accum_kernel(GridC g, int B, int W, const F *s, const F *T, const F *P, const double *h2,
+    kernel_accum_kernel(GridC g, int B, int W, int M, const F *s, const F *T, const F *P, const double *h2,
                         const double *cost, double *Ks, double *Kxi, double *Keta) {
     __shared__ F tot[8][6][33];
     const long long warp = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const int segs = (g.np + 31) / 32;
+    const int segs = (g.np + M - 1) / M;
     if (warp >= (long long)g.nr * g.nt * segs) return;      // whole warps: no block barrier below
-    const int k0 = (int)(warp % segs) * 32;
+    const int k0 = (int)(warp % segs) * M;
     const long long ij = warp / segs;
     const int j = (int)(ij % g.nt), i = (int)(ij / g.nt);
     const F idt = (F)(1.0 / g.dt), idp = (F)(1.0 / g.dp);
@@ -515,7 +518,7 @@ __global__ void __launch_bounds__(256)
     const long long st = (long long)g.np * B, sp = B;
     const long long ot_hi = j < g.nt - 1 ? st : 0, ot_lo = j > 0 ? st : 0;
     const int G = 32 / W, q = lane / W, l = lane - q * W;
-    const int nk = min(32, g.np - k0);
+    const int nk = min(M, g.np - k0);
     for (int m0 = 0; m0 < nk; m0 += G) {
         const int m = m0 + q;
         CompSum<F> sP, sX, sE;
@@ -727,21 +730,30 @@ cudaError_t run_misfit_table(int B, int n_rec, const double *tab, const double *
 template <typename F>
 cudaError_t run_kernel_accum(const GridC &g, int B, const void *s, const void *T, const void *P,
                              const double *h2, const double *cost, double *Ks, double *Kxi,
-                             double *Keta, cudaStream_t st) {
+                             double *Keta, int n_sm, cudaStream_t st) {
     // 16-byte loads where every row of the fields holds whole aligned vectors
     const bool vec = sizeof(F) == 4 && B % 4 == 0 && (size_t)T % 16 == 0 && (size_t)P % 16 == 0;
     const int per = vec ? (B + 3) / 4 : B;
     int W = 1;
     while (W < 32 && W < per) W *= 2;
-    const long long warps = (long long)g.nr * g.nt * ((g.np + 31) / 32);
+    // Nodes of a warp: a row in equal parts of at most 32, and in more where that leaves fewer than 12
+    // warps an SM (48 in FP64, whose terms keep the pipe busy beside the fixed part). ms with a
+    // warp per node / parts of 32 / now: 61x81x33 x 255 FP32 0.34 / 0.51 / 0.31, 21^3 x 255 FP32 0.071
+    // / 0.093 / 0.060, 11^3 x 4095 FP32 0.086 / 0.364 / 0.081, 11^3 x 4096 FP64 0.77 / 3.4 / 0.65.
+    const long long rows = (long long)g.nr * g.nt, least = (sizeof(F) == 8 ? 48LL : 12LL) * n_sm;
+    const int G = 32 / W;
+    long long segs = (g.np + 31) / 32;
+    if (rows * segs < least) segs = std::min((long long)(g.np + G - 1) / G, (least + rows - 1) / rows);
+    const int M = (int)((g.np + segs - 1) / segs + G - 1) / G * G;
+    const long long warps = rows * ((g.np + M - 1) / M);
     const unsigned blocks = blocks_for(warps * 32, 256);
     if constexpr (sizeof(F) == 4)
         if (vec) {
-            kernel_accum_kernel<F, 4><<<blocks, 256, 0, st>>>(g, B, W, (const F *)s, (const F *)T,
+            kernel_accum_kernel<F, 4><<<blocks, 256, 0, st>>>(g, B, W, M, (const F *)s, (const F *)T,
                                                               (const F *)P, h2, cost, Ks, Kxi, Keta);
             return cudaGetLastError();
         }
-    kernel_accum_kernel<F, 1><<<blocks, 256, 0, st>>>(g, B, W, (const F *)s, (const F *)T,
+    kernel_accum_kernel<F, 1><<<blocks, 256, 0, st>>>(g, B, W, M, (const F *)s, (const F *)T,
                                                       (const F *)P, h2, cost, Ks, Kxi, Keta);
     return cudaGetLastError();
 }
@@ -770,7 +782,7 @@ cudaError_t run_kernel_accum(const GridC &g, int B, const void *s, const void *T
                                        double *, int *, cudaStream_t);                         \
     template cudaError_t run_kernel_accum<F>(const GridC &, int, const void *, const void *,   \
                                              const void *, const double *, const double *,     \
-                                             double *, double *, double *, cudaStream_t);
+                                             double *, double *, double *, int, cudaStream_t);
 TTGB_INST(float)
 TTGB_INST(double)
 #undef TTGB_INST

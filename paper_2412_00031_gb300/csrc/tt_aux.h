@@ -72,6 +72,6 @@ cudaError_t run_misfit_table(int B, int n_rec, const double *tab, const double *
 template <typename F>
 cudaError_t run_kernel_accum(const GridC &g, int B, const void *s, const void *T, const void *P,
                              const double *h2, const double *cost, double *Ks, double *Kxi,
-                             double *Keta, cudaStream_t st);
+                             double *Keta, int n_sm, cudaStream_t st);
 
 }  // namespace ttgb

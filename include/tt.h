@@ -163,6 +163,7 @@ typedef struct {
     long long node_sweeps;    /* node visits counted once per batch: nodes x 8 x max iterations */
     int iters_max;            /* largest per-source iteration count */
     int grid_blocks, block_threads;
+    int thread_sources;       /* sources that a thread of the sweep updates at each node */
     long long launches;       /* kernels this context has launched since it was created */
     double warm_ms;           /* forward: device time of the warm-start inference (opts.init = 2),
                                  0 otherwise */

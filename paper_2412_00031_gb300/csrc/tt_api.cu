@@ -446,6 +446,11 @@ int factor_slice(const GridC &g, int B, size_t es) {
     return slice < 32 ? 32 : slice;
 }
 
+// Bytes of its cache: in FP32 a last source without a partner takes a pair's place (t0_pair_kernel).
+size_t factor_bytes(const GridC &g, int slice, size_t es) {
+    return 4 * es * (size_t)g.N * (es == 4 ? (slice + 1) / 2 * 2 : slice);
+}
+
 size_t partial_bytes(const tt_ctx *ctx, int B, size_t es) {
     return 2 * es * (size_t)B * (size_t)(kMaxBarrierGroups * ctx->n_sm);
 }
@@ -459,7 +464,7 @@ template <typename F> tt_status work_from_ctx(tt_ctx *ctx, Work<F> &W, int B, in
     ENSURE(ctx->tabT, sizeof(Vec2<F>) * (size_t)g.nt * B);
     ENSURE(ctx->tabP, sizeof(Vec2<F>) * (size_t)g.np * B);
     ENSURE(ctx->rec, sizeof(NodeRec<F>) * (size_t)g.N);
-    ENSURE(ctx->t0c, sizeof(Vec4<F>) * (size_t)g.N * slice);
+    ENSURE(ctx->t0c, factor_bytes(g, slice, sizeof(F)));
     ENSURE(ctx->partial, partial_bytes(ctx, B, sizeof(F)));
     ENSURE(ctx->conv, sizeof(int) * (size_t)B);
     ENSURE(ctx->iters, sizeof(int) * (size_t)B);
@@ -750,6 +755,7 @@ tt_status enq_forward(tt_ctx *ctx, Work<F> &W, const tt_model *m, int B, void *d
         CK(launch_refill_setup<F>(a, ctx->st));
         CK(launch_refill<F>(a, gblocks * groups, block, ctx->st));
         ctx->stats[TT_STATS_FORWARD].block_threads = block;
+        ctx->stats[TT_STATS_FORWARD].thread_sources = kFwdSourcesPerLane;
         ctx->launches += 2;
         max_grid_used = gblocks * groups;
     }
@@ -759,14 +765,16 @@ tt_status enq_forward(tt_ctx *ctx, Work<F> &W, const tt_model *m, int B, void *d
         a.src_n = n;
         int grid = 0;
         if (sched == 1 || n < 32) {  // a tile task stages 32 sources: short slices use planes
-            int block = 0, kernels = 0;
+            PlaneLaunch pl;
             const cudaError_t e = run_plane_forward<F>(a, o->fwd_groups, W.moved, ctx->n_sm,
-                                                       o->launch_blocks, &grid, &block, &kernels, ctx->st);
+                                                       o->launch_blocks, &pl, ctx->st);
             if (e == cudaErrorInvalidConfiguration)
                 return fail(ctx, TT_EINVAL, "slice of %d sources exceeds one resident launch", n);
             CK(e);
-            ctx->stats[TT_STATS_FORWARD].block_threads = block;
-            ctx->launches += kernels;
+            ctx->stats[TT_STATS_FORWARD].block_threads = pl.block;
+            ctx->stats[TT_STATS_FORWARD].thread_sources = pl.thread_sources;
+            ctx->launches += pl.kernels;
+            grid = pl.grid;
         } else {
             int per_sm = forward_tiled_blocks_per_sm<F>(sched - 2, B);
             if (per_sm <= 0) return fail(ctx, TT_ECUDA, "tiled sweep cannot be resident");
@@ -791,6 +799,7 @@ tt_status enq_forward(tt_ctx *ctx, Work<F> &W, const tt_model *m, int B, void *d
             CK(launch_t0_cache<F>(a, ctx->st));
             CK(launch_forward_tiled<F>(map_tau, map_rec, map_t0c, a, sched - 2, grid, ctx->st));
             ctx->stats[TT_STATS_FORWARD].block_threads = kTileThreads;
+            ctx->stats[TT_STATS_FORWARD].thread_sources = 1;
             ctx->launches += 2;
         }
         if (grid > max_grid_used) max_grid_used = grid;
@@ -868,7 +877,7 @@ tt_status enq_adjoint(tt_ctx *ctx, Work<F> &W, const tt_model *m, int B, const v
     // Face-coefficient sweep when the per-(node, source) coefficients fit the workspace
     // budget; otherwise the sweep that evaluates the flux velocities at every update.
     const bool faces = W.coef_ok;
-    int grid = 0, block = 0, slots = 0;
+    int grid = 0, block = 0, slots = 0, per_thread = 1;
     if (!faces && (s = sweep_shape<F>(ctx, B, ctx->full, o->launch_blocks, grid, block, slots)) != TT_OK)
         return s;
     const GeoTab<F> &t = geo<F>(ctx);
@@ -914,15 +923,16 @@ tt_status enq_adjoint(tt_ctx *ctx, Work<F> &W, const tt_model *m, int B, const v
         for (int q = 0; q < B; q += chunk) {
             a.src_lo = q;
             a.src_n = chunk < B - q ? chunk : B - q;
-            int gr = 0, bl = 0;
+            PlaneLaunch pl;
             const cudaError_t e = run_plane_adjoint<F>(a, o->adj_groups, W.partial, ctx->n_sm,
-                                                       o->launch_blocks, &gr, &bl, ctx->st);
+                                                       o->launch_blocks, &pl, ctx->st);
             if (e == cudaErrorInvalidConfiguration)
                 return fail(ctx, TT_EINVAL, "batch of %d sources exceeds one resident launch", B);
             CK(e);
-            grid = gr > grid ? gr : grid;
-            block = bl > block ? bl : block;
-            ctx->launches += 1;
+            grid = pl.grid > grid ? pl.grid : grid;
+            block = pl.block > block ? pl.block : block;
+            per_thread = pl.thread_sources > per_thread ? pl.thread_sources : per_thread;
+            ctx->launches += pl.kernels;
         }
     } else {
         CK(launch_adjoint<F>(a, grid, block, ctx->st));
@@ -931,6 +941,7 @@ tt_status enq_adjoint(tt_ctx *ctx, Work<F> &W, const tt_model *m, int B, const v
     CK(record(ctx, ctx->ev_stop[TT_STATS_ADJOINT]));
     ctx->stats[TT_STATS_ADJOINT].grid_blocks = grid;
     ctx->stats[TT_STATS_ADJOINT].block_threads = block;
+    ctx->stats[TT_STATS_ADJOINT].thread_sources = per_thread;
     return TT_OK;
 }
 
@@ -1681,10 +1692,10 @@ tt_status forward_tele_impl(tt_ctx *ctx, const tt_model *m, int n_ev, void *d_T,
     a.spin_ns = spin_ns(o);
     a.src_lo = 0;
     a.src_n = n_ev;
-    int grid = 0, block = 0, kernels = 0;
+    PlaneLaunch pl;
     CK(record(ctx, ctx->ev_start[TT_STATS_FORWARD]));
     const cudaError_t le = run_plane_forward<F>(a, o->fwd_groups, (int *)ctx->fwd_moved.p, ctx->n_sm,
-                                                o->launch_blocks, &grid, &block, &kernels, ctx->st);
+                                                o->launch_blocks, &pl, ctx->st);
     if (le == cudaErrorInvalidConfiguration)
         return fail(ctx, TT_EINVAL, "%d events exceed one resident launch", n_ev);
     CK(le);
@@ -1726,8 +1737,9 @@ tt_status forward_tele_impl(tt_ctx *ctx, const tt_model *m, int n_ev, void *d_T,
     S.node_updates = upd;
     S.node_sweeps = 8LL * imax * inner;
     S.iters_max = imax;
-    S.grid_blocks = grid;
-    S.block_threads = block;
+    S.grid_blocks = pl.grid;
+    S.block_threads = pl.block;
+    S.thread_sources = pl.thread_sources;
     if (left)
         return fail(ctx, TT_ENOTCONVERGED,
                     "tt_forward_tele: %d of %d events did not converge in %d iterations", left,
@@ -2378,7 +2390,7 @@ template <typename F> tt_status plan_alloc(tt_plan *p, Work<F> &W) {
     TTGB_GET(tabT, sizeof(Vec2<F>) * (size_t)g.nt * B);
     TTGB_GET(tabP, sizeof(Vec2<F>) * (size_t)g.np * B);
     TTGB_GET(rec, sizeof(NodeRec<F>) * (size_t)g.N);
-    TTGB_GET(t0c, sizeof(Vec4<F>) * (size_t)g.N * W.t0c_slice);
+    TTGB_GET(t0c, factor_bytes(g, W.t0c_slice, sizeof(F)));
     if (W.coef_ok) TTGB_GET(coef, coef_bytes);
     TTGB_GET(partial, partial_bytes(ctx, B, sizeof(F)));
     TTGB_GET(conv_f, sizeof(int) * B);

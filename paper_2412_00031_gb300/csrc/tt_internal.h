@@ -121,11 +121,14 @@ struct PlaneShape {
     int start[8], steps;
     int *moved;          // [3][src_n], by iteration mod 3: the source has not converged
 };
+// What a plane sweep launched: blocks, threads of a block, sources of a thread, kernels in all.
+struct PlaneLaunch {
+    int grid = 0, block = 0, thread_sources = 0, kernels = 0;
+};
 // The sources [src_lo, src_lo + src_n) of a; groups: barrier groups (0 = 1); moved: 3 * src_n ints.
-// grid, block and kernels receive the launch's shape and the number of kernels launched.
 template <typename F>
-cudaError_t run_plane_forward(FwdArgs<F> a, int groups, int *moved, int n_sm, int launch_blocks, int *grid,
-                              int *block, int *kernels, cudaStream_t st);
+cudaError_t run_plane_forward(FwdArgs<F> a, int groups, int *moved, int n_sm, int launch_blocks,
+                              PlaneLaunch *launch, cudaStream_t st);
 template <typename F> int refill_blocks_per_sm(int block, size_t smem, bool idx32, int scheme);
 template <typename F> cudaError_t launch_t0_cache(const FwdArgs<F> &a, cudaStream_t st);
 // Slot table of the retire-and-refill mode: slot s < n_slots takes source s.
@@ -157,7 +160,7 @@ template <typename F> cudaError_t launch_adjoint_coefs(const AdjArgs<F> &a, cuda
 // The sweep from the coefficients (tt_plane.cu) for the sources [src_lo, src_lo + src_n) of a; emax:
 // 6 * src_n values of F. cudaErrorInvalidConfiguration: they exceed one resident launch.
 template <typename F>
-cudaError_t run_plane_adjoint(AdjArgs<F> a, int groups, F *emax, int n_sm, int launch_blocks, int *grid,
-                              int *block, cudaStream_t st);
+cudaError_t run_plane_adjoint(AdjArgs<F> a, int groups, F *emax, int n_sm, int launch_blocks,
+                              PlaneLaunch *launch, cudaStream_t st);
 
 }  // namespace ttgb

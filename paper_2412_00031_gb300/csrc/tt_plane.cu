@@ -15,8 +15,8 @@
 //    they are set once after the solve (edge_kernel).
 //  - One block per SM and barrier group (run_plane_forward), threads over (node, source) without
 //    padding to whole warps of sources, consecutive warps on different SMs.
-//  - In large batches a thread holds two neighbouring sources: one load per stencil point, and
-//    packed FP32 arithmetic.
+//  - In large FP32 batches a thread holds two sources and updates them in packed arithmetic: two
+//    neighbours by one load per stencil point where rows are whole aligned pairs (Deal).
 //
 // Each update reads what it reads in the lexicographic order, so the bits are the same.
 //  - Threads are dealt to the sources that still iterate, anew every iteration.
@@ -106,7 +106,7 @@ struct Node {
     long long n;
 };
 
-template <typename F, int SCHEME, int NS>
+template <typename F, int SCHEME, int NS, int DEAL>
 __global__ void __launch_bounds__(kPlaneThreads, 1)
     plane_kernel(FwdArgs<F> a, PlaneShape m) {
     extern __shared__ int s_off[];             // plane offsets of the schedule
@@ -139,13 +139,19 @@ __global__ void __launch_bounds__(kPlaneThreads, 1)
     const unsigned nblk = (unsigned)m.grp_blocks;
     const long long osp = B, ost = (long long)g.np * B, osr = (long long)g.nt * g.np * B;
     using U = Update<F, SCHEME, NS>;
+    using D = Dealt<NS, DEAL>;
+    // Factors of a node: the launch's sources, one more for a pair where they are odd. Held for the
+    // Godunov updates (spills of pairs 106 -> 50 B; 121x161x161 x 256 sources, 3 iterations 250.6 -> 244.8
+    // ms), read from the arguments for pairs and single sources in LF (41^3 x 64 8.58 -> 8.42 ms).
+    constexpr bool kHeld = DEAL != kPairs || SCHEME == 1 || SCHEME == 2;
+    const int fac_row = D::units(a.src_n) * NS;
     const PlaneSched sch{s_off, s_start, a.nodes, a.n_planes, m.steps};
 
     for (int it = 0; it < a.max_iter; ++it) {
         // The sources that still iterate (NS to a thread), so that no thread is kept for converged
         // ones: a solve's last iterations have few sources, in any order of the batch.
         if (threadIdx.x < 32) {
-            const int n = plane_units<NS>(s_on, Bg / NS, s_list);
+            const int n = plane_units<NS, DEAL>(s_on, Bg, s_list);
             if (threadIdx.x == 0) s_units = n;
         }
         __syncthreads();
@@ -154,12 +160,13 @@ __global__ void __launch_bounds__(kPlaneThreads, 1)
         const int slots = (int)(((long long)m.grp_blocks * blockDim.x) / lanes);
         const bool any = tid < (long long)slots * lanes;
         const int slot = any ? (int)(tid / lanes) : 0;
-        const int bl = src0 + (any ? s_list[tid - (long long)slot * lanes] * NS : 0);
-        const int b = a.src_lo + bl;                                   // the thread's first source
-        const Vec4<F> *t0c = a.t0c + bl;
+        const int unit = any ? s_list[tid - (long long)slot * lanes] : 0;
+        const int bl = src0 + D::first(unit), off = D::step(unit, Bg);  // the thread's first source, the second's distance
+        const int b = a.src_lo + bl;
+        const Vec4<F> *t0c = a.t0c + (kHeld ? src0 + unit * NS : bl);
         bool act[NS];
 #pragma unroll
-        for (int h = 0; h < NS; ++h) act[h] = any && s_on[bl - src0 + h];
+        for (int h = 0; h < NS; ++h) act[h] = any && (h == 0 || off > 0) && s_on[bl - src0 + h * off];
         F err[NS];
 #pragma unroll
         for (int h = 0; h < NS; ++h) err[h] = 0;
@@ -193,14 +200,14 @@ __global__ void __launch_bounds__(kPlaneThreads, 1)
         auto load = [&]() {
             const Node d = place(o, pk);
             p = a.tau + (d.n * B + b);
-            ld_pack(p, v[0]);
-            ld_pack(p + osr, v[1]);
-            ld_pack(p - osr, v[2]);
-            ld_pack(p + ost, v[3]);
-            ld_pack(p - ost, v[4]);
-            ld_pack(p + osp, v[5]);
-            ld_pack(p - osp, v[6]);
-            fc = U::load(t0c + d.n * a.src_n);
+            ld_src<DEAL>(p, off, v[0]);
+            ld_src<DEAL>(p + osr, off, v[1]);
+            ld_src<DEAL>(p - osr, off, v[2]);
+            ld_src<DEAL>(p + ost, off, v[3]);
+            ld_src<DEAL>(p - ost, off, v[4]);
+            ld_src<DEAL>(p + osp, off, v[5]);
+            ld_src<DEAL>(p - osp, off, v[6]);
+            fc = U::load(t0c + d.n * (kHeld ? fac_row : a.src_n));
             rec = ld_rec(a.rec + d.n);
         };
         for (int tau = 0; tau < m.steps; ++tau) {
@@ -224,11 +231,7 @@ __global__ void __launch_bounds__(kPlaneThreads, 1)
                     if (x < total) pk = sch.entry(cp, x, o);
                     F tn[NS];
                     U::run(fc, v, rec, a.er, act, tn, err);
-                    // values that keep their bits are not stored: their line stays clean
-                    bool moved = false;
-#pragma unroll
-                    for (int h = 0; h < NS; ++h) moved = moved || bits_of(tn[h]) != bits_of(v[0][h]);
-                    if (moved) st_pack(p, tn);
+                    st_moved<DEAL>(p, off, tn, v[0]);
                     // a layer next to a face (second in the ordering: the entry face, last: the
                     // exit face) along some axis
                     if (SCHEME != 3 && (pkx & 0x40000000u)) {
@@ -237,10 +240,10 @@ __global__ void __launch_bounds__(kPlaneThreads, 1)
 #pragma unroll
                         for (int h = 0; h < NS; ++h) {
                             if (!act[h]) continue;
-                            const unsigned fx = s_fix[bl + h - src0];
+                            const unsigned fx = s_fix[bl + h * off - src0];
                             const int ci = (int)(fx >> 20), cj = (int)(fx >> 10) & 1023, ck = (int)fx & 1023;
                             auto put = [&](long long e, F x1, F x2, int fi, int fj, int fk) {
-                                if (!in_fixed_set(ci, cj, ck, fi, fj, fk)) p[e + h] = fmax_((F)2 * x1 - x2, x2);
+                                if (!in_fixed_set(ci, cj, ck, fi, fj, fk)) p[e + h * off] = fmax_((F)2 * x1 - x2, x2);
                             };
                             const F ua = rr ? v[1][h] : v[2][h], ub = rt ? v[3][h] : v[4][h], uc = rp ? v[5][h] : v[6][h];
                             const long long da = rr ? osr : -osr, db = rt ? ost : -ost, dc = rp ? osp : -osp;
@@ -268,7 +271,7 @@ __global__ void __launch_bounds__(kPlaneThreads, 1)
         int *flag = m.moved + (it % 3) * a.src_n;
 #pragma unroll
         for (int h = 0; h < NS; ++h)
-            if (act[h] && !(err[h] < a.tol)) flag[bl + h] = 1;
+            if (act[h] && !(err[h] < a.tol)) flag[bl + h * off] = 1;
         if (!grid_barrier(bar, a.spin_ns, nblk)) return;
         // every block takes the sources that have converged off its list; the group's first one
         // reports, and clears the flags of the iteration after the next
@@ -289,34 +292,37 @@ __global__ void __launch_bounds__(kPlaneThreads, 1)
     barrier_end(bar, nblk);
 }
 
-template <typename F, int NS> const void *plane_ptr(int scheme) {
+template <typename F, int NS, int DEAL> const void *plane_ptr(int scheme) {
     switch (scheme) {
-    case 0: return (const void *)plane_kernel<F, 0, NS>;
-    case 1: return (const void *)plane_kernel<F, 1, NS>;
-    case 2: return (const void *)plane_kernel<F, 2, NS>;
-    default: return (const void *)plane_kernel<F, 3, NS>;
+    case 0: return (const void *)plane_kernel<F, 0, NS, DEAL>;
+    case 1: return (const void *)plane_kernel<F, 1, NS, DEAL>;
+    case 2: return (const void *)plane_kernel<F, 2, NS, DEAL>;
+    default: return (const void *)plane_kernel<F, 3, NS, DEAL>;
     }
 }
 
-// The factor cache of pairs: (1/T0, u) of sources 2 q and 2 q + 1 interleaved (Fac2), the values
-// of t0_cache_kernel.
-__global__ void t0_pair_kernel(FwdArgs<float> a) {
+// The factor cache of two sources a thread: (1/T0, u) of a unit's sources interleaved (Fac2), the
+// values of t0_cache_kernel; for a unit of one source twice that one's.
+template <int DEAL> __global__ void t0_pair_kernel(FwdArgs<float> a, int grp_src) {
+    using D = Dealt<2, DEAL>;
     const GridC &g = a.g;
-    const int pairs = a.src_n / 2;
-    const long long total = g.N * pairs;
+    const int units = D::units(a.src_n);
+    const long long total = g.N * units;
     for (long long x = (long long)blockIdx.x * blockDim.x + threadIdx.x; x < total;
          x += (long long)gridDim.x * blockDim.x) {
-        const long long n = x / pairs;
-        const int b = a.src_lo + 2 * (int)(x - n * pairs);
+        const long long n = x / units;
+        const int u = (int)(x - n * units), src0 = 2 * u / grp_src * grp_src;   // grp_src is even
+        const int Bg = min(a.src_n, src0 + grp_src) - src0, ug = u - src0 / 2;
         const int k = (int)(n % g.np);
         const long long t = n / g.np;
         const int j = (int)(t % g.nt), i = (int)(t / g.nt);
         Vec4<float> c[2];
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
-            const SrcReg<float> S = load_src<float>(a.src, b + h, g.dr);
+            const int b = a.src_lo + src0 + D::first(ug) + h * D::step(ug, Bg);
+            const SrcReg<float> S = load_src<float>(a.src, b, g.dr);
             c[h].x = factor_T0<float>(S, i, __ldg(a.rad + i), __ldg(a.cost + j), __ldg(a.sint + j),
-                                      a.tabT[(long long)j * a.B + b + h], a.tabP[(long long)k * a.B + b + h],
+                                      a.tabT[(long long)j * a.B + b], a.tabP[(long long)k * a.B + b],
                                       g.flat != 0, c[h].y, c[h].z, c[h].w);
             if (in_fixed_set(S.ci, S.cj, S.ck, i, j, k)) c[h].x = -1.f;
         }
@@ -369,7 +375,7 @@ template <typename F> constexpr int kAdjThreads = sizeof(F) == 4 ? 1024 : kPlane
 // The adjoint sweep (Eq. 5) from the face coefficients (adj_coef_kernel, face_update), over every
 // node, in the same organisation; no faces to complete. emax: [3][2][src_n], by iteration mod 3 the
 // sources' largest |change| of P and, in the last ordering, largest |P|.
-template <typename F, int NS>
+template <typename F, int NS, int DEAL>
 __global__ void __launch_bounds__(kAdjThreads<F>, 1) adj_plane_kernel(AdjArgs<F> a, PlaneShape m, F *emax) {
     extern __shared__ __align__(8) int s_off[];
     __shared__ int s_units, s_start[8];
@@ -392,13 +398,14 @@ __global__ void __launch_bounds__(kAdjThreads<F>, 1) adj_plane_kernel(AdjArgs<F>
     const long long tid = ((long long)(threadIdx.x >> 5) * m.grp_blocks + blk) * 32 + (threadIdx.x & 31);
     BarrierState *bar = a.bar + grp;
     const unsigned nblk = (unsigned)m.grp_blocks;
+    using D = Dealt<NS, DEAL>;
     const long long sp = B, st = (long long)g.np * B, sr = (long long)g.nt * g.np * B;
     const long long plane = g.N * B;                               // coefficient plane stride
     const PlaneSched sch{s_off, s_start, a.nodes, a.n_planes, m.steps};
 
     for (int it = 0; it < a.max_iter; ++it) {
         if (threadIdx.x < 32) {
-            const int n = plane_units<NS>(s_on, Bg / NS, s_list);
+            const int n = plane_units<NS, DEAL>(s_on, Bg, s_list);
             if (threadIdx.x == 0) s_units = n;
         }
         for (int q = threadIdx.x; q < Bg; q += blockDim.x) s_err[q] = s_pm[q] = 0;
@@ -408,14 +415,15 @@ __global__ void __launch_bounds__(kAdjThreads<F>, 1) adj_plane_kernel(AdjArgs<F>
         const int slots = (int)(((long long)m.grp_blocks * blockDim.x) / lanes);
         const bool any = tid < (long long)slots * lanes;
         const int slot = any ? (int)(tid / lanes) : 0;
-        const int bl = src0 + (any ? s_list[tid - (long long)slot * lanes] * NS : 0);
+        const int unit = any ? s_list[tid - (long long)slot * lanes] : 0;
+        const int bl = src0 + D::first(unit), off = D::step(unit, Bg);
         const int b = a.src_lo + bl;
         const F *cX = a.coef, *cY = a.coef + plane, *cZ = a.coef + 2 * plane, *cW = a.coef + 3 * plane;
         bool act[NS];
         F err[NS], pmax[NS];
 #pragma unroll
         for (int h = 0; h < NS; ++h) {
-            act[h] = any && s_on[bl - src0 + h];
+            act[h] = any && (h == 0 || off > 0) && s_on[bl - src0 + h * off];
             err[h] = pmax[h] = 0;
         }
         Planes cp, np;
@@ -431,11 +439,11 @@ __global__ void __launch_bounds__(kAdjThreads<F>, 1) adj_plane_kernel(AdjArgs<F>
             const int i = o & 4 ? g.nr - 1 - aa : aa, j = o & 2 ? g.nt - 1 - bb : bb, k = o & 1 ? g.np - 1 - cc : cc;
             x = node_index(g, i, j, k) * B + b;
             last = o == 7;
-            ld_pack(cW + x, w);
-            ld_pack(cX + x, cx);
-            ld_pack(cY + x, cy);
-            ld_pack(cZ + x, cz);
-            ld_pack(a.P + x, po);
+            ld_src<DEAL>(cW + x, off, w);
+            ld_src<DEAL>(cX + x, off, cx);
+            ld_src<DEAL>(cY + x, off, cy);
+            ld_src<DEAL>(cZ + x, off, cz);
+            ld_src<DEAL>(a.P + x, off, po);
             // no flux through the outer faces: zero coefficients and values there
             const bool hr = i < g.nr - 1, lr = i > 0, ht = j < g.nt - 1, lt = j > 0, hp = k < g.np - 1, lp = k > 0;
 #pragma unroll
@@ -444,15 +452,15 @@ __global__ void __launch_bounds__(kAdjThreads<F>, 1) adj_plane_kernel(AdjArgs<F>
 #pragma unroll
                 for (int q = 0; q < 6; ++q) Pn[q][h] = 0;
             }
-            if (lr) ld_pack(cX + x - sr, mx);
-            if (lt) ld_pack(cY + x - st, my);
-            if (lp) ld_pack(cZ + x - sp, mz);
-            if (hr) ld_pack(a.P + x + sr, Pn[0]);
-            if (lr) ld_pack(a.P + x - sr, Pn[1]);
-            if (ht) ld_pack(a.P + x + st, Pn[2]);
-            if (lt) ld_pack(a.P + x - st, Pn[3]);
-            if (hp) ld_pack(a.P + x + sp, Pn[4]);
-            if (lp) ld_pack(a.P + x - sp, Pn[5]);
+            if (lr) ld_src<DEAL>(cX + x - sr, off, mx);
+            if (lt) ld_src<DEAL>(cY + x - st, off, my);
+            if (lp) ld_src<DEAL>(cZ + x - sp, off, mz);
+            if (hr) ld_src<DEAL>(a.P + x + sr, off, Pn[0]);
+            if (lr) ld_src<DEAL>(a.P + x - sr, off, Pn[1]);
+            if (ht) ld_src<DEAL>(a.P + x + st, off, Pn[2]);
+            if (lt) ld_src<DEAL>(a.P + x - st, off, Pn[3]);
+            if (hp) ld_src<DEAL>(a.P + x + sp, off, Pn[4]);
+            if (lp) ld_src<DEAL>(a.P + x - sp, off, Pn[5]);
         };
         for (int tau = 0; tau < m.steps; ++tau) {
             const int total = cp.total();
@@ -467,7 +475,6 @@ __global__ void __launch_bounds__(kAdjThreads<F>, 1) adj_plane_kernel(AdjArgs<F>
                     q += slots;
                     if (q < total) pk = sch.entry(cp, q, o);
                     F pn[NS];
-                    bool moved = false;
 #pragma unroll
                     for (int h = 0; h < NS; ++h) {
                         pn[h] = po[h];
@@ -478,9 +485,8 @@ __global__ void __launch_bounds__(kAdjThreads<F>, 1) adj_plane_kernel(AdjArgs<F>
                             err[h] = fmax_(err[h], fabs(pn[h] - po[h]));
                             if (last) pmax[h] = fmax_(pmax[h], fabs(pn[h]));
                         }
-                        moved = moved || bits_of(pn[h]) != bits_of(po[h]);
                     }
-                    if (moved) st_pack(a.P + x, pn);
+                    st_moved<DEAL>(a.P + x, off, pn, po);
                     if (q >= total) break;
                     load();
                 }
@@ -494,8 +500,8 @@ __global__ void __launch_bounds__(kAdjThreads<F>, 1) adj_plane_kernel(AdjArgs<F>
 #pragma unroll
         for (int h = 0; h < NS; ++h)
             if (act[h]) {
-                atomic_max_nonneg(&s_err[bl - src0 + h], err[h]);
-                atomic_max_nonneg(&s_pm[bl - src0 + h], pmax[h]);
+                atomic_max_nonneg(&s_err[bl - src0 + h * off], err[h]);
+                atomic_max_nonneg(&s_pm[bl - src0 + h * off], pmax[h]);
             }
         __syncthreads();
         for (int q = threadIdx.x; q < Bg; q += blockDim.x)
@@ -527,36 +533,37 @@ __global__ void __launch_bounds__(kAdjThreads<F>, 1) adj_plane_kernel(AdjArgs<F>
 }  // namespace
 
 template <typename F>
-cudaError_t run_plane_forward(FwdArgs<F> a, int groups, int *moved, int n_sm, int launch_blocks, int *grid,
-                              int *block, int *kernels, cudaStream_t st) {
+cudaError_t run_plane_forward(FwdArgs<F> a, int groups, int *moved, int n_sm, int launch_blocks,
+                              PlaneLaunch *launch, cudaStream_t st) {
     cudaError_t e;
     const int n = a.src_n;
     const bool tele = a.scheme == 3;
     PlaneShape m;
     memset(&m, 0, sizeof m);
     plane_starts(m, a.na, a.nb, a.nc);
-    // pairs need FP32 and rows of whole aligned pairs
-    const bool pair = sizeof(F) == 4 && n % 2 == 0 && a.B % 2 == 0 && a.src_lo % 2 == 0 &&
-                      (size_t)a.tau % 8 == 0 && plane_pairs(m, a.na, a.nb, a.nc, n, n_sm);
-    const void *fn = plane_ptr<F, 1>(a.scheme);
+    const bool pair = n % 2 == 0 && a.B % 2 == 0 && a.src_lo % 2 == 0 && (size_t)a.tau % 8 == 0;
+    const bool two = sizeof(F) == 4 && plane_two(m, a.na, a.nb, a.nc, n, a.scheme, pair, n_sm);
+    const void *fn = plane_ptr<F, 1, kPairs>(a.scheme);
     if constexpr (sizeof(F) == 4)
-        if (pair) fn = plane_ptr<F, 2>(a.scheme);
+        if (two) fn = pair ? plane_ptr<F, 2, kPairs>(a.scheme) : plane_ptr<F, 2, kHalves>(a.scheme);
+    launch->thread_sources = two ? 2 : 1;
     const size_t smem = sizeof(int) * (a.n_planes + 1 + 2 * (size_t)n) + n;
-    if ((e = plane_shape(m, fn, smem, a.na, a.nb, a.nc, n, pair ? 2 : 1, groups, kPlaneThreads, n_sm, launch_blocks, grid, block)) != cudaSuccess)
+    if ((e = plane_shape(m, fn, smem, a.na, a.nb, a.nc, n, two ? 2 : 1, groups, kPlaneThreads, n_sm, launch_blocks, launch)) != cudaSuccess)
         return e;
-    *kernels = tele ? 1 : 4;
+    launch->kernels = tele ? 1 : 4;
     m.moved = moved;
     if ((e = cudaMemsetAsync(moved, 0, sizeof(int) * 3 * (size_t)n, st)) != cudaSuccess) return e;
     if (!tele) {
         if constexpr (sizeof(F) == 4)
-            if (pair) {
-                const long long q = (a.g.N * (n / 2) + 255) / 256;
-                t0_pair_kernel<<<(unsigned)std::min(q, 152LL * 16), 256, 0, st>>>(a);
+            if (two) {
+                const unsigned q = (unsigned)std::min((a.g.N * ((n + 1) / 2) + 255) / 256, 152LL * 16);
+                if (pair) t0_pair_kernel<kPairs><<<q, 256, 0, st>>>(a, m.grp_src);
+                else t0_pair_kernel<kHalves><<<q, 256, 0, st>>>(a, m.grp_src);
             }
-        if (!pair && (e = launch_t0_cache<F>(a, st)) != cudaSuccess) return e;
+        if (!two && (e = launch_t0_cache<F>(a, st)) != cudaSuccess) return e;
     }
     void *args[] = {&a, &m};
-    if ((e = cudaLaunchCooperativeKernel(fn, dim3(*grid), dim3(*block), args, smem, st)) != cudaSuccess) return e;
+    if ((e = cudaLaunchCooperativeKernel(fn, dim3(launch->grid), dim3(launch->block), args, smem, st)) != cudaSuccess) return e;
     if (!tele)
         for (int axis = 1; axis <= 2; ++axis) {
             const long long q = (axis == 1 ? 4LL * a.g.np : 4LL * (a.g.nr + a.g.nt - 2)) * n;
@@ -566,29 +573,31 @@ cudaError_t run_plane_forward(FwdArgs<F> a, int groups, int *moved, int n_sm, in
 }
 
 template <typename F>
-cudaError_t run_plane_adjoint(AdjArgs<F> a, int groups, F *emax, int n_sm, int launch_blocks, int *grid,
-                              int *block, cudaStream_t st) {
+cudaError_t run_plane_adjoint(AdjArgs<F> a, int groups, F *emax, int n_sm, int launch_blocks,
+                              PlaneLaunch *launch, cudaStream_t st) {
     cudaError_t e;
     const int n = a.src_n;
     PlaneShape m;
     memset(&m, 0, sizeof m);
     plane_starts(m, a.g.nr, a.g.nt, a.g.np);
-    const bool pair = sizeof(F) == 4 && n % 2 == 0 && a.B % 2 == 0 && a.src_lo % 2 == 0 &&
-                      (size_t)a.P % 8 == 0 && plane_pairs(m, a.g.nr, a.g.nt, a.g.np, n, n_sm);
-    const void *fn = (const void *)adj_plane_kernel<F, 1>;
+    const bool pair = n % 2 == 0 && a.B % 2 == 0 && a.src_lo % 2 == 0 && (size_t)a.P % 8 == 0;
+    const bool two = sizeof(F) == 4 && plane_two(m, a.g.nr, a.g.nt, a.g.np, n, kAdjointSolver, pair, n_sm);
+    const void *fn = (const void *)adj_plane_kernel<F, 1, kPairs>;
     if constexpr (sizeof(F) == 4)
-        if (pair) fn = (const void *)adj_plane_kernel<F, 2>;
+        if (two) fn = pair ? (const void *)adj_plane_kernel<F, 2, kPairs> : (const void *)adj_plane_kernel<F, 2, kApart>;
+    launch->thread_sources = two ? 2 : 1;
+    launch->kernels = 1;
     const size_t smem = sizeof(int) * (a.n_planes + 2 + (size_t)n) + 2 * sizeof(F) * (size_t)n + n;
-    if ((e = plane_shape(m, fn, smem, a.g.nr, a.g.nt, a.g.np, n, pair ? 2 : 1, groups, kAdjThreads<F>, n_sm, launch_blocks, grid, block)) != cudaSuccess)
+    if ((e = plane_shape(m, fn, smem, a.g.nr, a.g.nt, a.g.np, n, two ? 2 : 1, groups, kAdjThreads<F>, n_sm, launch_blocks, launch)) != cudaSuccess)
         return e;
     if ((e = cudaMemsetAsync(emax, 0, sizeof(F) * 6 * (size_t)n, st)) != cudaSuccess) return e;
     void *args[] = {&a, &m, &emax};
-    return cudaLaunchCooperativeKernel(fn, dim3(*grid), dim3(*block), args, smem, st);
+    return cudaLaunchCooperativeKernel(fn, dim3(launch->grid), dim3(launch->block), args, smem, st);
 }
 
-template cudaError_t run_plane_adjoint<float>(AdjArgs<float>, int, float *, int, int, int *, int *, cudaStream_t);
-template cudaError_t run_plane_adjoint<double>(AdjArgs<double>, int, double *, int, int, int *, int *, cudaStream_t);
-template cudaError_t run_plane_forward<float>(FwdArgs<float>, int, int *, int, int, int *, int *, int *, cudaStream_t);
-template cudaError_t run_plane_forward<double>(FwdArgs<double>, int, int *, int, int, int *, int *, int *, cudaStream_t);
+template cudaError_t run_plane_adjoint<float>(AdjArgs<float>, int, float *, int, int, PlaneLaunch *, cudaStream_t);
+template cudaError_t run_plane_adjoint<double>(AdjArgs<double>, int, double *, int, int, PlaneLaunch *, cudaStream_t);
+template cudaError_t run_plane_forward<float>(FwdArgs<float>, int, int *, int, int, PlaneLaunch *, cudaStream_t);
+template cudaError_t run_plane_forward<double>(FwdArgs<double>, int, int *, int, int, PlaneLaunch *, cudaStream_t);
 
 }  // namespace ttgb

@@ -6,6 +6,7 @@
 #include <cstring>
 
 #include "tt_internal.h"
+#include "tt_update.cuh"
 
 namespace ttgb {
 
@@ -63,15 +64,64 @@ struct PlaneSched {
     }
 };
 
-// list = the units of NS sources of which one is on, in order; returns their number. One warp.
-template <int NS> __device__ __forceinline__ int plane_units(const unsigned char *on_, int units, int *list) {
+// How a thread holds its sources of a group of n.
+enum Deal {
+    kPairs,    // one, or two neighbours (2 u and 2 u + 1) by vector accesses: rows of whole aligned pairs
+    kHalves,   // u and u + (n + 1) / 2, scalar accesses, coalesced like a single source's; any n, any place
+    kApart,    // two neighbours by scalar accesses; any n, any place
+};
+template <int NS, int DEAL> struct Dealt {
+    static_assert(NS == 2 || DEAL == kPairs, "");
+    static __device__ __forceinline__ int units(int n) { return (n + NS - 1) / NS; }
+    static __device__ __forceinline__ int first(int u) { return DEAL == kHalves ? u : u * NS; }
+    // distance of a unit's second source from its first; 0: there is none (the last unit of an odd n)
+    static __device__ __forceinline__ int step(int u, int n) {
+        if (DEAL == kPairs) return 1;
+        const int d = DEAL == kHalves ? (n + 1) / 2 : 1;
+        return first(u) + d < n ? d : 0;
+    }
+};
+
+// The field values at p of a thread's sources; off: Dealt's step.
+template <int DEAL, typename F, int NS>
+__device__ __forceinline__ void ld_src(const F *p, int off, F (&v)[NS]) {
+    if constexpr (DEAL != kPairs) {
+        v[0] = p[0];
+        v[1] = p[off];
+    } else {
+        ld_pack(p, v);
+    }
+}
+// v to p where its bits differ from those of old: a line of values that all stay is not made dirty
+template <int DEAL, typename F, int NS>
+__device__ __forceinline__ void st_moved(F *p, int off, const F (&v)[NS], const F (&old)[NS]) {
+    bool moved[NS], any = false;
+#pragma unroll
+    for (int h = 0; h < NS; ++h) {
+        moved[h] = bits_of(v[h]) != bits_of(old[h]);
+        any = any || moved[h];
+    }
+    if constexpr (DEAL != kPairs) {
+        if (moved[0]) p[0] = v[0];
+        if (moved[1]) p[off] = v[1];
+    } else if (any) {
+        st_pack(p, v);
+    }
+}
+
+// list = the units of sources of which one is on, in order; returns their number. One warp.
+template <int NS, int DEAL> __device__ __forceinline__ int plane_units(const unsigned char *on_, int n_src, int *list) {
+    using D = Dealt<NS, DEAL>;
+    const int units = D::units(n_src);
     int n = 0;
     const int lane = threadIdx.x & 31;
     for (int u0 = 0; u0 < units; u0 += 32) {
         const int u = u0 + lane;
         bool on = false;
-#pragma unroll
-        for (int h = 0; h < NS; ++h) on = on || (u < units && on_[u * NS + h]);
+        if (u < units) {
+            on = on_[D::first(u)];
+            if (NS == 2) on = on || on_[D::first(u) + D::step(u, n_src)];
+        }
         const unsigned mask = __ballot_sync(0xffffffffu, on);
         if (on) list[n + __popc(mask & ((1u << lane) - 1u))] = u;
         n += __popc(mask);
@@ -94,12 +144,25 @@ inline void plane_starts(PlaneShape &m, int na, int nb, int nc) {
     m.steps = m.start[7] + planes;
 }
 
-// Pairs of sources where a time step has more updates than the GPU holds threads: half the
-// instructions and loads an update. Below that a thread per source has the shorter time step.
-// Forward LF, ms per 2 iterations, single / pairs: 81^3 x 16 sources 6.81 / 6.97, x 32 8.32 /
-// 7.86, x 100 14.2 / 12.1; 121x161x161 x 32 26.6 / 23.0.
-inline bool plane_pairs(const PlaneShape &m, int na, int nb, int nc, int n, int n_sm) {
-    return 8.0 * na * nb * nc / m.steps * n > (double)kPlaneThreads * n_sm;
+// Two sources a thread where a time step has more updates than a line times the SMs: half the
+// instructions and packed arithmetic an update; below it a thread per source has the shorter step. The
+// line of pairs: the threads of an SM. Forward LF, ms per 2 iterations, single / pairs: 81^3 x 16
+// sources 6.81 / 6.97, x 32 8.32 / 7.86, x 100 14.2 / 12.1; 121x161x161 x 32 26.6 / 23.0.
+// A batch or field that does not have whole aligned pairs deals its sources otherwise (scalar
+// accesses, so the line lies higher), in the adjoint as neighbours (its rows come from DRAM: 3
+// iterations at 121x161x161 x 111 single / halves / apart 116 / 126 / 99 ms). Around the lines, ms of
+// 6 iterations in LF, 3 in the others, single / two (updates a step and SM):
+//   LF          121x161x161 x 15 57.4 / 59.3 (1107), 41^3 x 255 15.4 / 14.7 (1458)
+//   Godunov     121x161x161 x 47 72.8 / 73.2 (3468), 81^3 x 199 47.1 / 46.3 (4669)
+//   isotropic   41x61x67 x 255 21.5 / 21.9 (2407), 121x161x161 x 47 69.3 / 67.2 (3468)
+//   teleseismic 81x101x101 x 23 138 / 129 (696, a whole solve)
+//   adjoint     41^3 x 255 9.4 / 9.1 (1611), 121x161x161 x 23 40.7 / 42.9 (1746), x 31 48.2 / 44.6 (2354)
+// At 121x161x161 x 255: LF 361 -> 256, Godunov 291 -> 250, adjoint 234 -> 194 (256: 244, 245, 174).
+constexpr int kAdjointSolver = -1;
+inline bool plane_two(const PlaneShape &m, int na, int nb, int nc, int n, int solver, bool pairs, int n_sm) {
+    const int line = pairs || solver == 3 ? kPlaneThreads
+                     : solver == 0 ? 1300 : solver == 1 ? 2600 : solver == 2 ? 3500 : 2000;
+    return n > 1 && 8.0 * na * nb * nc / m.steps * n > (double)line * n_sm;
 }
 
 // Blocks, threads and barrier groups (0 = 1) for n sources, ns to a thread; smem: dynamic shared
@@ -107,7 +170,7 @@ inline bool plane_pairs(const PlaneShape &m, int na, int nb, int nc, int n, int 
 // barrier of 608 blocks takes 2.5 us, of 152 1.6 us); no more threads than the widest plane has
 // nodes and sources. cudaErrorInvalidConfiguration: the sources exceed one resident launch.
 inline cudaError_t plane_shape(PlaneShape &m, const void *fn, size_t smem, int na, int nb, int nc, int n, int ns,
-                               int groups, int max_threads, int n_sm, int launch_blocks, int *grid, int *block) {
+                               int groups, int max_threads, int n_sm, int launch_blocks, PlaneLaunch *launch) {
     cudaError_t e;
     if ((e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess)
         return e;
@@ -119,7 +182,7 @@ inline cudaError_t plane_shape(PlaneShape &m, const void *fn, size_t smem, int n
     long long widest = 0;
     for (int x = 0; x < 3; ++x)
         for (int y = x + 1; y < 3; ++y) widest = std::max(widest, (long long)ext[x] * ext[y]);
-    const long long want = (widest * (n / ns) / groups / n_sm + 31) / 32 * 32;
+    const long long want = (widest * ((n + ns - 1) / ns) / groups / n_sm + 31) / 32 * 32;
     if (want < threads) threads = want < 32 ? 32 : (int)want;
     int per_sm = 0;
     if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, threads, smem)) != cudaSuccess) return e;
@@ -132,11 +195,11 @@ inline cudaError_t plane_shape(PlaneShape &m, const void *fn, size_t smem, int n
     groups = (n + m.grp_src - 1) / m.grp_src;
     m.grp_blocks = most / groups;
     // a group's blocks hold at least one thread per source
-    const int need = (m.grp_src / ns + threads - 1) / threads;
+    const int need = ((m.grp_src + ns - 1) / ns + threads - 1) / threads;
     if (m.grp_blocks < need) m.grp_blocks = need;
     if ((long long)m.grp_blocks * groups > (long long)per_sm * n_sm) return cudaErrorInvalidConfiguration;
-    *grid = m.grp_blocks * groups;
-    *block = threads;
+    launch->grid = m.grp_blocks * groups;
+    launch->block = threads;
     return cudaSuccess;
 }
 

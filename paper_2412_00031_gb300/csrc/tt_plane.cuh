@@ -146,22 +146,27 @@ inline void plane_starts(PlaneShape &m, int na, int nb, int nc) {
 
 // Two sources a thread where a time step has more updates than a line times the SMs: half the
 // instructions and packed arithmetic an update; below it a thread per source has the shorter step. The
-// line of pairs: the threads of an SM. Forward LF, ms per 2 iterations, single / pairs: 81^3 x 16
-// sources 6.81 / 6.97, x 32 8.32 / 7.86, x 100 14.2 / 12.1; 121x161x161 x 32 26.6 / 23.0.
-// A batch or field that does not have whole aligned pairs deals its sources otherwise (scalar
-// accesses, so the line lies higher), in the adjoint as neighbours (its rows come from DRAM: 3
-// iterations at 121x161x161 x 111 single / halves / apart 116 / 126 / 99 ms). Around the lines, ms of
-// 6 iterations in LF, 3 in the others, single / two (updates a step and SM):
-//   LF          121x161x161 x 15 57.4 / 59.3 (1107), 41^3 x 255 15.4 / 14.7 (1458)
-//   Godunov     121x161x161 x 47 72.8 / 73.2 (3468), 81^3 x 199 47.1 / 46.3 (4669)
-//   isotropic   41x61x67 x 255 21.5 / 21.9 (2407), 121x161x161 x 47 69.3 / 67.2 (3468)
-//   teleseismic 81x101x101 x 23 138 / 129 (696, a whole solve)
-//   adjoint     41^3 x 255 9.4 / 9.1 (1611), 121x161x161 x 23 40.7 / 42.9 (1746), x 31 48.2 / 44.6 (2354)
+// line depends on the solver (Godunov pairs spill) and on how the sources are dealt: a batch or field
+// without whole aligned pairs takes scalar accesses, in halves or, in the adjoint, as neighbours (its
+// rows come from DRAM: 3 iterations at 121x161x161 x 111 single / halves / apart 116 / 126 / 99 ms).
+// Single / two beside the lines, ms of 6 iterations in LF, 3 in the others (updates a step and SM):
+//   LF pairs         41^3 x 96 10.1 / 10.2 (549), 41^3 x 128 10.9 / 10.7 (732), 81^3 x 64 31.0 / 29.0
+//   LF halves        121x161x161 x 15 57.4 / 59.3 (1107), 41^3 x 255 15.4 / 14.7 (1458)
+//   Godunov pairs    41x61x67 x 256 22.5 / 23.2 (2416), 121x161x161 x 40 65.6 / 64.4 (2951)
+//   Godunov halves   41^3 x 699 21.6 / 21.9 (3997), 41x61x67 x 511 37.0 / 35.6 (4823)
+//   isotropic pairs  41^3 x 384 13.5 / 13.5 (2196), 121x161x161 x 32 52.4 / 51.7 (2361)
+//   isotropic halves 41x61x67 x 255 21.3 / 21.6 (2407), 81^3 x 127 32.4 / 31.6 (2980)
+//   teleseismic      81x101x101 x 23, a whole solve, halves 138 / 129 (696)
+//   adjoint pairs    81^3 x 24 11.4 / 11.8 (592), 81^3 x 32 13.4 / 12.4 (789)
+//   adjoint apart    121x161x161 x 23 40.7 / 42.9 (1746), x 31 48.2 / 44.6 (2354)
 // At 121x161x161 x 255: LF 361 -> 256, Godunov 291 -> 250, adjoint 234 -> 194 (256: 244, 245, 174).
 constexpr int kAdjointSolver = -1;
 inline bool plane_two(const PlaneShape &m, int na, int nb, int nc, int n, int solver, bool pairs, int n_sm) {
-    const int line = pairs || solver == 3 ? kPlaneThreads
-                     : solver == 0 ? 1300 : solver == 1 ? 2600 : solver == 2 ? 3500 : 2000;
+    const int line = solver == 0   ? (pairs ? kPlaneThreads : 1300)
+                     : solver == 1 ? (pairs ? 2300 : 2900)
+                     : solver == 2 ? (pairs ? 2900 : 4300)
+                     : solver == 3 ? kPlaneThreads
+                                   : (pairs ? kPlaneThreads : 2000);
     return n > 1 && 8.0 * na * nb * nc / m.steps * n > (double)line * n_sm;
 }
 

@@ -11,7 +11,7 @@ import tt_inputs as I
 pytestmark = pytest.mark.gpu
 
 # updates of a time step and SM from which on a thread holds two sources, by solver
-LINE = {"lf": 1300, "iso": 2600, "aniso": 3500, "tele": 768, "adj": 2000}
+LINE = {"lf": 1300, "iso": 2900, "aniso": 4300, "tele": 768, "adj": 2000}
 
 
 def _steps(na, nb, nc):
@@ -130,6 +130,26 @@ def test_adjoint(shape, max_iter):
                            tt.default_opts(tt.TT_F32, max_iter_adj=max_iter, **kw), allow_unconverged=True)
         return P, it, tt.tt_get_stats(ctx, tt.TT_STATS_ADJOINT)["thread_sources"]
     _check(solve, n, VARIANTS + [(1, 0, dict(adj_groups=3)), (0, 0, dict(adj_groups=3))])
+    ctx.close()
+
+
+@pytest.mark.parametrize("kind,scheme,below,above", [("lf", 0, 550, 1000), ("iso", 1, 2000, 2600), ("aniso", 2, 2500, 3200)])
+def test_even_batches_on_both_sides_of_the_line(kind, scheme, below, above):
+    """A Godunov thread holds a pair only from larger batches on than an LF one; the bits do not tell."""
+    import torch
+    import paper_2412_00031_gb300 as tt
+    shape = (26, 27, 29)
+    per = _batch(kind, shape) / (1.2 * LINE[kind])
+    n, m = (int(x * per) // 2 * 2 for x in (above, below))
+    w, src = _case(kind, shape, n)
+    model = tuple(torch.as_tensor(np.ascontiguousarray(a), dtype=torch.float32, device="cuda") for a in (w.s, w.xi, w.eta))
+    ctx = tt.tt_ctx_create(w.grid.as_dict())
+    tau = []
+    for k, want in ((n, 2), (m, 1)):
+        tau.append(_field(shape, k, 0))
+        tt.tt_forward(ctx, model, src[:k], tau[-1], None, tt.default_opts(tt.TT_F32, scheme=scheme))
+        assert tt.tt_get_stats(ctx)["thread_sources"] == want
+    assert torch.equal(tau[0][..., :m], tau[1])
     ctx.close()
 
 

@@ -27,7 +27,7 @@
 // together in tensor memory. So a tile takes three slab copies, not nine. The copies had bound the
 // layers: a TMA copy of 128 short rows runs at about one row per two clocks and SM whatever the
 // rows' width (layer 1 took as long as the others), and there were nine per tile. Tiles do not cross
-// a plane's end, which wastes less than a tile per plane. The order of an accumulator's sums
+// a plane's end, which wastes less than a tile per plane; small planes of several grids share one. The order of an accumulator's sums
 // (di, dj, channels) is that of a tile by itself, so the bits are the same.
 // Measured: the warm start of 32 sources at 121x161x161 (network on every other node) 7.63 ms with
 // nine copies a tile, 4.11 ms so.
@@ -246,9 +246,10 @@ struct RowGeo {
     int R;              // rows of one grid: n_r Si
     int wins;           // windows of 126 rows of a plane: ceil(Si / 126)
     int chunks;         // runs of planes that a window is cut into
+    int gb, rb;         // grids of a tile and rows of each: 1 and 128, or small planes side by side
 };
 
-// A CTA's work: window win of the output planes [i0, i1) of grid g. Neighbouring windows run at
+// A CTA's work: window win of the output planes [i0, i1) of the gb grids from g on. Neighbouring windows run at
 // the same time on neighbouring CTAs, so that a row's three dj reads meet in L2.
 struct Walk {
     int g, win, i0, i1;
@@ -258,10 +259,15 @@ __device__ __forceinline__ Walk walk_of(const RowGeo &G, long long T) {
     w.win = (int)(T % G.wins);
     const long long t = T / G.wins;
     const int c = (int)(t % G.chunks);
-    w.g = (int)(t / G.chunks);
+    w.g = (int)(t / G.chunks) * G.gb;
     w.i0 = (int)((long long)G.nr * c / G.chunks);
     w.i1 = (int)((long long)G.nr * (c + 1) / G.chunks);
     return w;
+}
+
+// Grid groups, and walks of a launch.
+__host__ __device__ __forceinline__ long long walks(const RowGeo &G) {
+    return (long long)((G.nb + G.gb - 1) / G.gb) * G.chunks * G.wins;
 }
 
 __device__ __forceinline__ bool pad_row(const RowGeo &G, int n) {
@@ -325,7 +331,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     __syncthreads();
     tc_fence_after();
     const unsigned tmem = *s_tmem;
-    const long long total = (long long)G.nb * G.chunks * G.wins;
+    const long long total = walks(G);
 
     if (warp == 0) {
         if (lane == 0) {
@@ -334,11 +340,12 @@ __global__ void __launch_bounds__(kThreads, 1)
             int s = 0;
             unsigned ph = 0, armed = 0, armed_par = 0;
             bool ok = true;
+            const unsigned stage_bytes = 3u * (unsigned)(G.gb * G.rb) * L::ROW;
             for (long long T = blockIdx.x; ok && T < total; T += gridDim.x) {
                 const Walk w = walk_of(G, T);
                 for (int p = w.i0 - 1; p <= w.i1; ++p) {
                     if (!bar_wait(empty(s), ph ^ 1u, limit, s_abort)) { ok = false; break; }
-                    bar_expect_tx(full(s), L::STAGE);
+                    bar_expect_tx(full(s), stage_bytes);
                     const int r0 = p * G.Si + w.win * kTileStep - 1;
                     for (int dj = 0; dj < 3; ++dj)
                         tma_rows(sA + s * L::STAGE + dj * L::SLAB, &map, r0 + (dj - 1) * G.Sj, w.g, full(s));
@@ -409,13 +416,14 @@ __global__ void __launch_bounds__(kThreads, 1)
 #pragma unroll
         for (int c = 0; c < (FINAL ? 1 : 32); ++c) bz[c] = MODE == kEpiGate ? 0.0f : bias[c];
         float *ex = exch + a * 4 * 2 * 2 * 32;
+        const int mg = m / G.rb, mr = m - mg * G.rb;             // grid of the tile and row of its window
         int u = -1, par = 0;                                     // accumulator and group of the next tile
         unsigned uph = 0;
         bool ok = true;
         for (long long T = blockIdx.x; ok && T < total; T += gridDim.x) {
             const Walk wk = walk_of(G, T);
-            const int g = wk.g, rw = wk.win * kTileStep + m;       // the thread's row of the plane
-            const bool out_ok = m < kTileStep && rw < G.Si;
+            const int g = wk.g + mg, rw = wk.win * kTileStep + mr;  // the thread's grid and row of the plane
+            const bool out_ok = mr < G.rb - 2 && mg < G.gb && g < G.nb && rw < G.Si;
             const int j = rw / G.Sj, k = rw - j * G.Sj;
             const bool zero = !out_ok || k == G.np || j >= G.nt;    // padding rows are written as zero
             for (int i = wk.i0; i < wk.i1; ++i) {
@@ -853,15 +861,15 @@ PFN_cuTensorMapEncodeTiled_v12000 map_encoder() {
 }
 
 // Tensor map over rows of 8 KC BF16 channels: dims (channels, R rows, nb grids); a box is
-// box_rows rows of one grid, swizzled as the descriptors expect.
-cudaError_t encode_rows(CUtensorMap *map, const void *base, const RowGeo &G, int KC,
-                        int box_rows = kTileRows) {
+// box_rows rows of box_grids grids, swizzled as the descriptors expect.
+cudaError_t encode_rows(CUtensorMap *map, const void *base, const RowGeo &G, int KC, int box_rows,
+                        int box_grids = 1) {
     PFN_cuTensorMapEncodeTiled_v12000 enc = map_encoder();
     if (!enc) return cudaErrorNotSupported;
     const cuuint64_t row = (cuuint64_t)KC * 16;
     cuuint64_t dims[3] = {(cuuint64_t)KC * 8, (cuuint64_t)G.R, (cuuint64_t)G.nb};
     cuuint64_t strides[2] = {row, row * (cuuint64_t)G.R};
-    cuuint32_t box[3] = {(cuuint32_t)KC * 8, (cuuint32_t)box_rows, 1};
+    cuuint32_t box[3] = {(cuuint32_t)KC * 8, (cuuint32_t)box_rows, (cuuint32_t)box_grids};
     cuuint32_t estr[3] = {1, 1, 1};
     const CUresult r = enc(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void *>(base), dims,
                            strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
@@ -876,7 +884,7 @@ int walk_chunks(const RowGeo &G, int n_sm) {
     int best = 1;
     long long least = -1;
     for (int c = 1; c <= G.nr; ++c) {
-        const long long waves = ((long long)G.nb * G.wins * c + n_sm - 1) / n_sm;
+        const long long waves = (walks(G) * c + n_sm - 1) / n_sm;   // G.chunks is 1 here
         const long long cost = waves * ((G.nr + c - 1) / c + 1);
         if (least < 0 || cost < least) {
             least = cost;
@@ -891,7 +899,7 @@ cudaError_t launch_layer(const void *in, RowGeo G, const __nv_bfloat16 *wimg,
                          const float *bias, void *out, int n_sm, int *err,
                          unsigned long long limit, cudaStream_t st, const void *gate = nullptr) {
     CUtensorMap map;
-    cudaError_t e = encode_rows(&map, in, G, KC);
+    cudaError_t e = encode_rows(&map, in, G, KC, G.rb, G.gb);
     if (e != cudaSuccess) return e;
     G.chunks = walk_chunks(G, n_sm);
     // more than half the shared memory of an SM: one CTA per SM, which owns its TMEM
@@ -899,7 +907,7 @@ cudaError_t launch_layer(const void *in, RowGeo G, const __nv_bfloat16 *wimg,
     const void *fn = (const void *)conv3d_tc_kernel<KC, NO, MODE>;
     e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
-    const long long total = (long long)G.nb * G.chunks * G.wins;
+    const long long total = walks(G);
     const unsigned grid = (unsigned)(total < n_sm ? total : n_sm);
     conv3d_tc_kernel<KC, NO, MODE><<<grid, kThreads, smem, st>>>(
         map, G, reinterpret_cast<const uint4 *>(wimg), bias, reinterpret_cast<const uint4 *>(gate),
@@ -945,6 +953,13 @@ RowGeo row_geo(const ConvDims &d) {
     G.R = d.D * G.Si;
     G.wins = (G.Si + kTileStep - 1) / kTileStep;
     G.chunks = 1;
+    // Planes of at most 62 rows: those of two to four grids in one tile (two rows more of each for the
+    // dk taps), as a plane by itself leaves most of the tile empty. Inference in tiles across the
+    // planes' ends, with nine copies each / a plane a tile / so: 256 grids of 121x4x4 nodes 0.458 /
+    // 0.792 / 0.263 ms, 1024 of 61x5x5 1.150 / 1.512 / 0.619.
+    const bool small = 2 * (G.Si + 2) <= kTileRows && G.nb > 1;
+    G.gb = small ? kTileRows / (G.Si + 2) : 1;
+    G.rb = small ? G.Si + 2 : kTileRows;
     return G;
 }
 

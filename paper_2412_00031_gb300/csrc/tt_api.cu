@@ -1859,9 +1859,13 @@ tt_status tt_mgrid_expand(tt_ctx *ctx, const tt_mgrid *mg, const double *d_G, do
     MgTabs tb;
     tt_status s;
     if ((s = mgrid_tables(ctx, mg, d, tb)) != TT_OK) return s;
-    ENSURE(ctx->mg_scr, sizeof(double) * (size_t)d.H * d.nr * d.nt * d.cp);
-    CK(run_mgrid_expand(d, d_G, tb.lo, tb.Wr, tb.Wt, tb.Wp, (double *)ctx->mg_scr.p, d_D, ctx->st));
-    ctx->launches += 2;
+    // Two steps through rows of coarse nodes while these are few against the forward nodes, and at most
+    // 1 GiB. ms at 101x201x201, one step / two: 5 grids, 11 coarse nodes along phi 0.70 / 0.16, 150 0.70
+    // / 0.59, 200 0.70 / 0.75; one grid, 200 0.20 / 0.17, 400 0.20 / 0.29, 4096 0.20 / 2.62.
+    const size_t rows = sizeof(double) * (size_t)d.H * d.nr * d.nt * d.cp;
+    const bool two = d.cp <= d.np * (0.8 + 0.45 / d.H) && rows <= 1ull << 30 && grow(ctx->mg_scr, rows);
+    CK(run_mgrid_expand(d, d_G, tb.lo, tb.Wr, tb.Wt, tb.Wp, two ? (double *)ctx->mg_scr.p : nullptr, d_D, ctx->st));
+    ctx->launches += two ? 2 : 1;
     return TT_OK;
 }
 

@@ -195,6 +195,8 @@ __global__ void project_r_kernel(MgDims d, const double *__restrict__ T2,
 // products G W_r W_t around the row (i, j), / H; then D[i][j][k] = sum over h of the two products
 // E W_p around the node. With the eight products per grid formed at every node the FP64 pipe
 // took 0.7 ms at 101x201x201 and 5 grids; the rows hold np / cp times fewer values than the nodes.
+// DIRECT forms the eight products at the node, where the rows hold as many values as the nodes or
+// would not fit.
 __global__ void expand_rows_kernel(MgDims d, const double *__restrict__ G, const int *__restrict__ lo,
                                    const double *__restrict__ Wr, const double *__restrict__ Wt,
                                    double *__restrict__ E) {
@@ -216,22 +218,39 @@ __global__ void expand_rows_kernel(MgDims d, const double *__restrict__ G, const
     E[q] = e / d.H;
 }
 
-__global__ void expand_kernel(MgDims d, const double *__restrict__ E, const int *__restrict__ lo,
-                              const double *__restrict__ Wp, double *D) {
+template <bool DIRECT>
+__global__ void expand_kernel(MgDims d, const double *__restrict__ E, const double *__restrict__ G,
+                              const int *__restrict__ lo, const double *__restrict__ Wr,
+                              const double *__restrict__ Wt, const double *__restrict__ Wp, double *D) {
     const long long n = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     const long long N = (long long)d.nr * d.nt * d.np;
     if (n >= N) return;
     const int k = (int)(n % d.np);
     const long long ij = n / d.np;
-    const int *lop = lo + (long long)d.H * (d.nr + d.nt);
+    const int i = (int)(ij / d.nt), j = (int)(ij - (long long)i * d.nt);
+    const int *lor = lo, *lot = lo + (long long)d.H * d.nr, *lop = lot + (long long)d.H * d.nt;
     double acc = 0.0;
     for (int h = 0; h < d.H; ++h) {
         const int c0 = lop[h * d.np + k];
-        const double *e = E + ((long long)h * d.nr * d.nt + ij) * d.cp + c0;
         const double *w = Wp + ((long long)h * d.cp + c0) * d.np + k;
-        acc += e[0] * w[0] + e[1] * w[d.np];
+        const double w0 = w[0], w1 = w[d.np];
+        if constexpr (DIRECT) {
+            const int a0 = lor[h * d.nr + i], b0 = lot[h * d.nt + j];
+            double sh = 0.0;
+            for (int a = a0; a < a0 + 2; ++a) {
+                const double wr = Wr[((long long)h * d.cr + a) * d.nr + i];
+                for (int b = b0; b < b0 + 2; ++b) {
+                    const double *g = G + (((long long)h * d.cr + a) * d.ct + b) * d.cp + c0;
+                    sh += wr * Wt[((long long)h * d.ct + b) * d.nt + j] * (g[0] * w0 + g[1] * w1);
+                }
+            }
+            acc += sh;
+        } else {
+            const double *e = E + ((long long)h * d.nr * d.nt + ij) * d.cp + c0;
+            acc += e[0] * w0 + e[1] * w1;
+        }
     }
-    D[n] = acc;
+    D[n] = DIRECT ? acc / d.H : acc;
 }
 
 // max |x| of each of three FP64 fields: per-block maxima, then one block over them.
@@ -379,8 +398,13 @@ cudaError_t run_mgrid_project(const MgDims &d, const double *K, const double *h2
 cudaError_t run_mgrid_expand(const MgDims &d, const double *G, const int *lo, const double *Wr,
                              const double *Wt, const double *Wp, double *E, double *D,
                              cudaStream_t st) {
+    const unsigned nb = nblocks((long long)d.nr * d.nt * d.np, 256);
+    if (!E) {
+        expand_kernel<true><<<nb, 256, 0, st>>>(d, nullptr, G, lo, Wr, Wt, Wp, D);
+        return cudaGetLastError();
+    }
     expand_rows_kernel<<<nblocks((long long)d.H * d.nr * d.nt * d.cp, 256), 256, 0, st>>>(d, G, lo, Wr, Wt, E);
-    expand_kernel<<<nblocks((long long)d.nr * d.nt * d.np, 256), 256, 0, st>>>(d, E, lo, Wp, D);
+    expand_kernel<false><<<nb, 256, 0, st>>>(d, E, G, lo, Wr, Wt, Wp, D);
     return cudaGetLastError();
 }
 

@@ -35,7 +35,7 @@ cudaError_t run_mgrid_project(const MgDims &d, const double *K, const double *h2
                               const double *Wt, const double *Wp, const int *rng, double *T1,
                               double *T2, double *G, cudaStream_t st);
 // Eq. 15: D at the forward nodes from the coefficients G; lo = the three axes' lo tables; E
-// ([H][nr][nt][cp]) is scratch.
+// ([H][nr][nt][cp]) is scratch, or NULL: one step without it.
 cudaError_t run_mgrid_expand(const MgDims &d, const double *G, const int *lo, const double *Wr,
                              const double *Wt, const double *Wp, double *E, double *D,
                              cudaStream_t st);

@@ -55,3 +55,27 @@ def test_a_few_coarse_nodes_do_not_take_longer_than_many():
         return best
     assert ms(3) <= 1.3 * ms(11)
     ctx.close()
+
+
+def test_short_hats_do_not_take_longer_than_long_ones_of_as_many_values():
+    """Five grids of 11 x 11 x 200 against 11 x 11 x 100 at 101x201x201: twice the outputs, of hats of two
+    nodes; 2.0 times the time with an unrolled remainder, 1.6 without."""
+    import torch
+    import paper_2412_00031_gb300 as tt
+    shape = (101, 201, 201)
+    ctx = tt.tt_ctx_create(_grid(shape))
+    K = torch.randn(shape, dtype=torch.float64, device="cuda")
+
+    def ms(cp):
+        G = torch.zeros((5, 11, 11, cp), dtype=torch.float64, device="cuda")
+        best = np.inf
+        for _ in range(10):
+            a, b = (torch.cuda.Event(enable_timing=True) for _ in range(2))
+            a.record()
+            tt.tt_mgrid_project(ctx, tt.mgrid(11, 11, cp, 5), K, G)
+            b.record()
+            torch.cuda.synchronize()
+            best = min(best, a.elapsed_time(b))
+        return best
+    assert ms(200) <= 1.8 * ms(100)
+    ctx.close()

@@ -347,7 +347,7 @@ def gpu_arm(args, rank, world):
         "config": workload_config(w, world),
         "step_form": ("one captured CUDA graph per step (tt_plan)" if args.plan
                       else "four C-ABI calls per step"),
-        "roofline": {"bound": "hbm", "kernel": "plane_kernel<float, 0, 2>", "achieved": f_gbs,
+        "roofline": {"bound": "hbm", "kernel": "plane_kernel<float, 0, 2, 0>", "achieved": f_gbs,
                      "peak": hbm, "peak_kind": peak_kind, "unit": "GB/s", "frac": f_gbs / hbm,
                      "traffic": traffic, "algorithmic_bytes_per_launch": f_bytes,
                      "launch_ms": f_ms, "kernel_source_digest": digest},
@@ -460,7 +460,7 @@ def godunov_leg(args, gp, world):
     fwd_kernel = hbm_kernel(f_ms, float(np.mean([s["node_updates"] for s in fwd])),
                             float(np.mean([s["node_sweeps"] for s in fwd])),
                             FWD_BYTES_PER_UPDATE, FWD_BYTES_PER_NODE_SWEEP, hbm)
-    fwd_kernel["kernel"] = "plane_kernel<float, 2, 2>"
+    fwd_kernel["kernel"] = "plane_kernel<float, 2, 2, 0>"
     # The same forward from tau = 1 (opts.init = 0), for comparison with the start from above.
     o1 = tt.default_opts(tt.TT_F32, scheme=2, fwd_groups=gp.opts.fwd_groups)
     it1 = tt.tt_forward(gp.ctx, gp.model, gp.w.src, gp.tau, None, o1)
@@ -881,7 +881,7 @@ def tele_leg(args):
                                    "%dx%d over 400 km x %g deg (FP64); region 121x161x161 "
                                    "anisotropic (FP32)" % (n_ev, n_r, n_d, dmax)},
             "tol_fwd_region_s": 3e-5,
-            "note": "region solve: one persistent launch of the node-hyperplane sweep (Lax-"
+            "note": "region solve: one persistent launch of the plane sweep (Lax-"
                     "Friedrichs on T, faces fixed, FP32 arithmetic, convergence on the device)"}
 
 

@@ -1647,7 +1647,7 @@ tt_status tt_tele_region_times(tt_ctx *ctx, int dtype, int n_r, int n_d, double 
 namespace {
 
 // The region's solve of teleseismic events (R17): one persistent cooperative launch of the
-// node-hyperplane sweep with SCHEME 3 (Lax-Friedrichs on T itself, faces held fixed), the
+// plane sweep (tt_plane.cu) with SCHEME 3 (Lax-Friedrichs on T itself, faces held fixed), the
 // events as the batch, each stopping on its own criterion inside the launch.
 template <typename F>
 tt_status forward_tele_impl(tt_ctx *ctx, const tt_model *m, int n_ev, void *d_T,

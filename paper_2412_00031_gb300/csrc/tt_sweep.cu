@@ -1,12 +1,13 @@
-// Persistent fast-sweeping kernels of libttgb: the factored Lax-Friedrichs forward sweep
-// (Eq. "4", Sec. 3.1) and the upwind adjoint sweep (Eq. 5), both run hyperplane by
-// hyperplane (Sec. 3.4) inside one cooperative launch per solve.
+// Persistent fast-sweeping kernels of libttgb beside the plane sweeps (tt_plane.cu): the forward
+// sweep with retire-and-refill (opts.fwd_slots) and on tile hyperplanes (opts.sweep_schedule 2 to 4),
+// the adjoint that forms its flux velocities at every update (when the face coefficients do not fit),
+// and the factor cache and face coefficients that the plane sweeps read.
 //
-// Work mapping. Batched fields are stored [node][source]. Thread t of the launch owns one
-// source b = t mod B for the whole solve and a slot t / B; on each hyperplane the slots
-// stride over the plane's nodes. With B >= 32 a warp reads 32 consecutive sources of one
-// node, so every field access is a coalesced 128-byte line and the per-node model values
-// are warp-wide broadcasts. Between hyperplanes the launch crosses a bounded grid barrier.
+// Work mapping. Batched fields are stored [node][source]. A solve is one cooperative launch whose
+// threads own sources for the whole solve and take the nodes of each hyperplane (Sec. 3.4) in
+// slots; a warp reads consecutive sources of one node, so every field access is coalesced and the
+// per-node model values are warp-wide broadcasts. Between hyperplanes a barrier group of blocks
+// crosses a bounded grid barrier.
 #include <cuda.h>
 #include <cuda_runtime.h>
 

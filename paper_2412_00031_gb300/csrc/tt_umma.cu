@@ -27,8 +27,9 @@
 // together in tensor memory. So a tile takes three slab copies, not nine. The copies had bound the
 // layers: a TMA copy of 128 short rows runs at about one row per two clocks and SM whatever the
 // rows' width (layer 1 took as long as the others), and there were nine per tile. Tiles do not cross
-// a plane's end, which wastes less than a tile per plane; small planes of several grids share one. The order of an accumulator's sums
-// (di, dj, channels) is that of a tile by itself, so the bits are the same.
+// a plane's end, which wastes less than a tile per plane; small planes of several grids share one
+// (row_geo). The order of an accumulator's sums (di, dj, channels) is that of a tile by itself, so
+// the bits are the same.
 // Measured: the warm start of 32 sources at 121x161x161 (network on every other node) 7.63 ms with
 // nine copies a tile, 4.11 ms so.
 //
@@ -406,8 +407,8 @@ __global__ void __launch_bounds__(kThreads, 1)
             bar_drain(drain, 0, limit);
         }
     } else {
-        // epilogue group a (warps 2-5: a = 0, warps 6-9: a = 1) takes this CTA's tiles of
-        // parity a, in accumulator buffer a; warp w reads TMEM lanes 32 (w % 4) ...
+        // epilogue group a (warps 2-5: a = 0, warps 6-9: a = 1) takes every other tile of this
+        // CTA, in the accumulators of the ring as they come; warp w reads TMEM lanes 32 (w % 4) ...
         const int a = (warp - 2) >> 2;
         const int quarter = warp & 3;
         const int m = quarter * 32 + lane;

@@ -141,8 +141,8 @@ __global__ void __launch_bounds__(kPlaneThreads, 1)
     using U = Update<F, SCHEME, NS>;
     using D = Dealt<NS, DEAL>;
     // Factors of a node: the launch's sources, one more for a pair where they are odd. Held for the
-    // Godunov updates (spills of pairs 106 -> 50 B; 121x161x161 x 256 sources, 3 iterations 250.6 -> 244.8
-    // ms), read from the arguments for pairs and single sources in LF (41^3 x 64 8.58 -> 8.42 ms).
+    // Godunov updates (spills of pairs 106 -> 50 B; 121x161x161 x 256 sources, 3 iterations 252 -> 248 ms),
+    // read from the arguments in LF (41^3 x 64, 6 iterations 8.58 -> 8.40).
     constexpr bool kHeld = DEAL != kPairs || SCHEME == 1 || SCHEME == 2;
     const int fac_row = D::units(a.src_n) * NS;
     const PlaneSched sch{s_off, s_start, a.nodes, a.n_planes, m.steps};
@@ -163,7 +163,10 @@ __global__ void __launch_bounds__(kPlaneThreads, 1)
         const int unit = any ? s_list[tid - (long long)slot * lanes] : 0;
         const int bl = src0 + D::first(unit), off = D::step(unit, Bg);  // the thread's first source, the second's distance
         const int b = a.src_lo + bl;
-        const Vec4<F> *t0c = a.t0c + (kHeld ? src0 + unit * NS : bl);
+        const Vec4<F> *t0c;
+        if constexpr (kHeld && NS == 2) t0c = a.t0c + (src0 + unit * NS);
+        else if constexpr (kHeld && sizeof(F) == 4) t0c = a.t0c + src0 + unit;   // fewer registers: x 1 source 48.8 -> 47.2 ms
+        else t0c = a.t0c + bl;
         bool act[NS];
 #pragma unroll
         for (int h = 0; h < NS; ++h) act[h] = any && (h == 0 || off > 0) && s_on[bl - src0 + h * off];
@@ -207,7 +210,8 @@ __global__ void __launch_bounds__(kPlaneThreads, 1)
             ld_src<DEAL>(p - ost, off, v[4]);
             ld_src<DEAL>(p + osp, off, v[5]);
             ld_src<DEAL>(p - osp, off, v[6]);
-            fc = U::load(t0c + d.n * (kHeld ? fac_row : a.src_n));
+            if constexpr (kHeld) fc = U::load(t0c + d.n * fac_row);
+            else fc = U::load(t0c + d.n * a.src_n);
             rec = ld_rec(a.rec + d.n);
         };
         for (int tau = 0; tau < m.steps; ++tau) {

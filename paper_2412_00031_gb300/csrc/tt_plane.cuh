@@ -11,8 +11,8 @@
 namespace ttgb {
 
 // Threads of an SM: 80 registers a thread. Fewer threads of more registers are slower, also where
-// they would not spill (the Godunov updates): 121x161x161 x 256 sources 639 / 543 / 494 / 482 ms
-// with 384 / 512 / 640 / 768.
+// they would not spill (the Godunov updates): 121x161x161 x 256 sources, a whole solve with 384 / 512 /
+// 640 / 768 threads 547 / 464 / 429 / 408 ms, Lax-Friedrichs 4163 / 3458 / 3068 / 2852.
 constexpr int kPlaneThreads = 768;
 
 // NS neighbouring sources of one node: one load or store.

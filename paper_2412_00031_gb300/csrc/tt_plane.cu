@@ -21,7 +21,7 @@
 // Each update reads what it reads in the lexicographic order, so the bits are the same.
 //  - Threads are dealt to the sources that still iterate, anew every iteration.
 // Measured, ms of a solve, with a barrier per plane and 456 or 608 blocks / now (one GB300):
-// 41^3 x 1 source FP64 352 / 64; 121x161x161 x 1 (Godunov) 107 / 47; 67x83x95 x 37 378 / 212;
+// 41^3 x 1 source FP64 352 / 55; 121x161x161 x 1 (Godunov) 107 / 47; 67x83x95 x 37 378 / 214;
 // 81^3 x 64 353 / 231; 101x141x151 x 112 1377 / 1197; 121x161x161 x 256 (Godunov) 483 / 423,
 // (Lax-Friedrichs, in the order of the last counts) 2643 / 2644;
 // 81x101x101 x 24 events 430 / 189. Of a time step's 4 us at 81^3 x 64 the barrier and the schedule

@@ -490,7 +490,7 @@ def refill_leg(args, dev, world, slots, gp):
     model = (f32(big.s), f32(big.xi), f32(big.eta))
     ctx = tt.tt_ctx_create(big.grid.as_dict())
     tau = torch.empty(big.grid.shape + (big.n_src,), dtype=torch.float32, device=dev)
-    o_refill = tt.default_opts(tt.TT_F32, fwd_slots=slots, fwd_groups=gp.opts.fwd_groups)
+    o_refill = tt.default_opts(tt.TT_F32, fwd_slots=slots)   # the groups tuned for the step are not its own
     o_batch = tt.default_opts(tt.TT_F32, fwd_groups=gp.opts.fwd_groups)
     starts = list(range(0, big.n_src, slots))
     taus = [torch.empty(big.grid.shape + (min(slots, big.n_src - s0),), dtype=torch.float32,

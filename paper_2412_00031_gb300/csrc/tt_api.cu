@@ -1969,7 +1969,8 @@ tt_status autotune_impl(tt_ctx *ctx, const tt_model *m, const tt_point *h_src, i
     std::vector<int> it(B);
     // c = -1, untimed, for the Godunov solvers: it leaves the sources' counts, so that every candidate
     // runs in the batch order of repeated calls (the first one would run in the given order).
-    for (int c = opts->scheme == 0 ? 0 : -1; c < kTuneCandidates; ++c) {
+    const bool ordered = B >= 64 && opts->fwd_order == 0 && opts->fwd_slots == 0;
+    for (int c = opts->scheme != 0 && ordered ? -1 : 0; c < kTuneCandidates; ++c) {
         tt_opts o = *opts;
         o.init = 0;
         // Lax-Friedrichs: two iterations show the per-iteration cost. The Godunov solvers

@@ -21,9 +21,9 @@
 // Each update reads what it reads in the lexicographic order, so the bits are the same.
 //  - Threads are dealt to the sources that still iterate, anew every iteration.
 // Measured, ms of a solve, with a barrier per plane and 456 or 608 blocks / now (one GB300):
-// 41^3 x 1 source FP64 352 / 55; 121x161x161 x 1 (Godunov) 107 / 47; 67x83x95 x 37 378 / 214;
-// 81^3 x 64 353 / 231; 101x141x151 x 112 1377 / 1197; 121x161x161 x 256 (Godunov) 483 / 423,
-// (Lax-Friedrichs, in the order of the last counts) 2643 / 2644;
+// 41^3 x 1 source FP64 352 / 55; 121x161x161 x 1 (Godunov) 107 / 42-47; 67x83x95 x 37 378 / 214;
+// 81^3 x 64 353 / 231; 101x141x151 x 112 1377 / 1197; 121x161x161 x 256, in the order of the last
+// counts, Godunov 483 / 400, Lax-Friedrichs 2643 / 2540-2560;
 // 81x101x101 x 24 events 430 / 189. Of a time step's 4 us at 81^3 x 64 the barrier and the schedule
 // take 2.2; at 101x141x151 x 112 it is 7.5 us, four rounds of loads and updates of 1.3 us each.
 // Measured and not kept: loading the next node's factors ahead (also across the barrier), an L2
@@ -161,11 +161,12 @@ __global__ void __launch_bounds__(kPlaneThreads, 1)
         const bool any = tid < (long long)slots * lanes;
         const int slot = any ? (int)(tid / lanes) : 0;
         const int unit = any ? s_list[tid - (long long)slot * lanes] : 0;
-        const int bl = src0 + D::first(unit), off = D::step(unit, Bg);  // the thread's first source, the second's distance
+        // the thread's first source and the second's distance from it
+        const int bl = src0 + D::first(unit), off = D::step(unit, Bg);
         const int b = a.src_lo + bl;
         const Vec4<F> *t0c;
         if constexpr (kHeld && NS == 2) t0c = a.t0c + (src0 + unit * NS);
-        else if constexpr (kHeld && sizeof(F) == 4) t0c = a.t0c + src0 + unit;   // fewer registers: x 1 source 48.8 -> 47.2 ms
+        else if constexpr (kHeld && sizeof(F) == 4) t0c = a.t0c + src0 + unit;   // fewer registers: 48.8 -> 47.2 ms x 1
         else t0c = a.t0c + bl;
         bool act[NS];
 #pragma unroll
